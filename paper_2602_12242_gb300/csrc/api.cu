@@ -211,6 +211,7 @@ const char* mx_kernel_name(const mx_ctx* ctx, int q) {
       if (ctx->plane) return dft ? "xik_dft_kernel" : "xik_kernel";
       return ctx->fast_x ? "xi_kernel" : "x_inv_kernel";
     case KID_YZ:
+      if (ctx->yz3) return "yz3_kernel";
       if (ctx->plane) return ctx->quad ? "yzq_kernel" : "yzh_kernel";
       return ctx->yz2d ? "yz2d_kernel" : "yz_fused_kernel";
     case KID_Y_FWD: return "y_fwd_kernel";
@@ -644,7 +645,7 @@ mx_status mx_demag_spectrum(mx_ctx* ctx, float* out, mx_stream_t stream) {
     set_error("mx_demag_spectrum: demag kernel not built");
     return MX_ERR_NOT_BUILT;
   }
-  if (ctx->plane) return plane_spectrum_out(ctx, out, (cudaStream_t)stream);
+  if (ctx->plane || ctx->yz3) return plane_spectrum_out(ctx, out, (cudaStream_t)stream);
   const long no = (long)ctx->g.Hx * ctx->g.Oy * ctx->g.Oz;
   MX_CUDA_TRY(cudaMemcpyAsync(out, ctx->nhat, sizeof(float) * 6 * no, cudaMemcpyDeviceToDevice,
                               (cudaStream_t)stream));

@@ -318,7 +318,10 @@ mx_status demag_setup(mx_ctx* ctx) {
 
 mx_status demag_yz(mx_ctx* ctx, cudaStream_t st) {
   const Grid& g = ctx->g;
-  if (ctx->yz2d) {
+  if (ctx->yz3) {
+    ProfScope ps(ctx, KID_YZ, st);
+    MX_TRY(yz3_pass(ctx, false, st, false));
+  } else if (ctx->yz2d) {
     ProfScope ps(ctx, KID_YZ, st);
     MX_TRY(yz2d_pass(ctx, st));
   } else if (ctx->fused_yz) {

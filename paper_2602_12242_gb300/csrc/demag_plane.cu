@@ -647,6 +647,12 @@ static mx_status yzh_pass(mx_ctx* ctx, cudaStream_t st, bool setup) {
   }
 }
 
+// The y/z passes of the plane path, w1 -> w2.
+static mx_status plane_yz(mx_ctx* ctx, cudaStream_t st) {
+  if (ctx->yz3) return yz3_pass(ctx, true, st, false);
+  return ctx->quad ? quad_pass(ctx, st, false) : yzh_pass(ctx, st, false);
+}
+
 mx_status plane_setup(mx_ctx* ctx) {
   MX_TRY(upload_w32());
   const int path = ctx->p.demag_path;
@@ -654,8 +660,12 @@ mx_status plane_setup(mx_ctx* ctx) {
                   xk_pass(ctx, nullptr, nullptr, false, nullptr, true) == MX_OK;
   // the four-CTA y/z kernel where it fits, else the two-CTA one
   // (MX_DEMAG_PLANE_PAIR forces the two-CTA kernel)
-  ctx->quad = xk && path != MX_DEMAG_PLANE_PAIR && quad_pass(ctx, nullptr, true) == MX_OK;
-  ctx->plane = ctx->quad || (xk && yzh_pass(ctx, nullptr, true) == MX_OK);
+  // the few-layer y/z kernel wherever it fits, in place on the small-grid
+  // layout unless the grid's x passes are the kx-major ones
+  ctx->yz3 = path == MX_DEMAG_AUTO && ctx->fast_x && yz3_pass(ctx, xk, nullptr, true) == MX_OK;
+  if (ctx->yz3 && !xk) ctx->fused_yz = true;
+  ctx->quad = xk && !ctx->yz3 && path != MX_DEMAG_PLANE_PAIR && quad_pass(ctx, nullptr, true) == MX_OK;
+  ctx->plane = ctx->quad || (xk && ctx->yz3) || (xk && yzh_pass(ctx, nullptr, true) == MX_OK);
   ctx->g.oct4 = ctx->quad ? 1 : 0;
   ctx->xlocal = ctx->plane && path == MX_DEMAG_PLANE_XLOCAL;
   clear_error();
@@ -686,7 +696,7 @@ mx_status plane_field(mx_ctx* ctx, const float4* m, float4* hd, cudaStream_t st)
   }
   {
     ProfScope ps(ctx, KID_YZ, st);
-    MX_TRY(ctx->quad ? quad_pass(ctx, st, false) : yzh_pass(ctx, st, false));
+    MX_TRY(plane_yz(ctx, st));
   }
   {
     ProfScope ps(ctx, KID_X_INV, st);
@@ -706,7 +716,7 @@ mx_status plane_stage_xlocal(mx_ctx* ctx, int mode, const StageIO& io, cudaStrea
   }
   {
     ProfScope ps(ctx, KID_YZ, st);
-    MX_TRY(ctx->quad ? quad_pass(ctx, st, false) : yzh_pass(ctx, st, false));
+    MX_TRY(plane_yz(ctx, st));
   }
   ProfScope ps(ctx, KID_X_INV_LOCAL, st);
   return xl_pass(ctx, mode, io, st);

@@ -43,6 +43,7 @@
 #include "fft.cuh"
 #include "kernels.cuh"
 #include "regfft.cuh"
+#include "zcol.cuh"
 
 namespace mx {
 
@@ -72,74 +73,6 @@ __device__ __forceinline__ void quad_inv_step2(float2* line, int s, const float2
     for (int t = 0; t < S; ++t) line[k1 + E * t] = v[j * S + t];
   }
   __syncwarp();
-}
-
-// (a, b, c) <- N (a, b, c) for the symmetric 3x3 tensor N, complex vectors.
-__device__ __forceinline__ void tensor_apply(float2& a, float2& b, float2& c, float nxx, float nyy, float nzz,
-                                             float nxy, float nxz, float nyz) {
-  const float2 mx = a, my = b, mz = c;
-  a = make_float2(fmaf(nxz, mz.x, fmaf(nxy, my.x, nxx * mx.x)), fmaf(nxz, mz.y, fmaf(nxy, my.y, nxx * mx.y)));
-  b = make_float2(fmaf(nyz, mz.x, fmaf(nyy, my.x, nxy * mx.x)), fmaf(nyz, mz.y, fmaf(nyy, my.y, nxy * mx.y)));
-  c = make_float2(fmaf(nzz, mz.x, fmaf(nyz, my.x, nxz * mx.x)), fmaf(nzz, mz.y, fmaf(nyz, my.y, nxz * mx.y)));
-}
-
-// Tensor multiply of one column's half spectrum, kz parity PAR: y[.][q] holds
-// kz = 2 q + PAR; kz and its mirror P - kz share one octant entry (the mirror
-// with N_xz and N_yz negated).  tq: the column's entry at qz = 0, qzs floats
-// per step of qz; sy = -1 where ky > Py/2 (N_xy and N_yz are odd in ky).
-template <int P, int PAR>
-__device__ __forceinline__ void quad_z_multiply(float2 (&y)[3][P / 2], const float* __restrict__ tq, long qzs,
-                                                float sy) {
-  constexpr int Q = P / 2;
-#pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const int kz = 2 * q + PAR;
-    if (kz > P / 2) continue;  // done with its mirror
-    const float2* t = reinterpret_cast<const float2*>(tq + kz * qzs);
-    const float2 t01 = __ldg(t), t23 = __ldg(t + 1), t45 = __ldg(t + 2);
-    const float nxy = sy * t23.y, nyz = sy * t45.y;
-    tensor_apply(y[0][q], y[1][q], y[2][q], t01.x, t01.y, t23.x, nxy, t45.x, nyz);
-    if (kz != 0 && kz != P / 2) {
-      const int qm = Q - q - PAR;  // 2 qm + PAR = P - kz
-      tensor_apply(y[0][qm], y[1][qm], y[2][qm], t01.x, t01.y, t23.x, nxy, -t45.x, -nyz);
-    }
-  }
-}
-
-// One column, kz parity p (uniform across the warp): half-length forward
-// transform of the nz planes of each component (times W_P^z first for odd
-// kz), the tensor multiply and the inverse half transform (times W_P^-z after
-// it for odd kz); y[c][n] is this parity's share of output plane n.  col: the
-// column's element in line 0 of the plane.
-template <int P>
-__device__ __forceinline__ void quad_z_column(const float2* col, int pitch, int nz, const float* __restrict__ tq,
-                                              long qzs, float sy, int p, float2 (&y)[3][P / 2]) {
-  constexpr int Q = P / 2;
-  constexpr int TS = 32 / P;  // W_P^n = c_w32[n TS]
-#pragma unroll
-  for (int c = 0; c < 3; ++c)
-#pragma unroll
-    for (int n = 0; n < Q; ++n) y[c][n] = n < nz ? col[(c * nz + n) * pitch] : make_float2(0.f, 0.f);
-  if (p) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int n = 1; n < Q; ++n) y[c][n] = cmul(y[c][n], c_w32[n * TS]);
-  }
-#pragma unroll
-  for (int c = 0; c < 3; ++c) RegFft<Q, false>::run(y[c]);
-  if (p)
-    quad_z_multiply<P, 1>(y, tq, qzs, sy);
-  else
-    quad_z_multiply<P, 0>(y, tq, qzs, sy);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) RegFft<Q, true>::run(y[c]);
-  if (p) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int n = 1; n < Q; ++n) y[c][n] = cmul(y[c][n], cconj(c_w32[n * TS]));
-  }
 }
 
 // barrier `id` (1..15) over `count` threads (whole warps)
@@ -294,7 +227,7 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kQuadNT, 2)
       const float* tq = nk + ((long)(qy & 3) * o4 + (qy >> 2)) * 6;
       float2* cp = plane + col;
       float2 y[3][Q];
-      quad_z_column<P>(cp, PITCH, nz, tq, qzs, fy ? -1.f : 1.f, p, y);
+      z_column<P>(cp, PITCH, nz, [&](int kz, int) { return z_entry(tq, qzs, kz); }, fy ? -1.f : 1.f, p, y);
       named_sync(bar, 64);  // both parities have read these columns
       if (p == 0) {
 #pragma unroll

@@ -43,6 +43,11 @@ mx_status fast_setup(mx_ctx* ctx);
 mx_status yz2d_pass(mx_ctx* ctx, cudaStream_t st);
 mx_status fast_x_pass(mx_ctx* ctx, const float4* m, float4* hd, bool inverse, cudaStream_t st);
 
+// demag_yz3.cu: the y/z passes of grids with few layers, in place on the
+// small-grid spectrum w1, or (km) w1 -> w2 on the kx-major ones of the plane
+// path (setup: check the grid fits and set the kernel's attributes)
+mx_status yz3_pass(mx_ctx* ctx, bool km, cudaStream_t st, bool setup);
+
 // demag_plane.cu
 mx_status plane_setup(mx_ctx* ctx);
 mx_status plane_field(mx_ctx* ctx, const float4* m, float4* hd, cudaStream_t st);

@@ -1,0 +1,43 @@
+"""Schedules of the demag convolution chosen by grid size, against the
+size-generic passes (which the oracle checks in test_gpu_parity.py).
+
+Tolerance: a schedule's field has about one FP32 rounding (6e-8 relative) per
+radix pass, at most 11 passes per axis and direction, so 66 in all, adding up
+in quadrature to 5e-7 of the field's norm; two schedules then differ by 7e-7.
+2e-6 leaves a factor of three.
+"""
+import numpy as np
+import pytest
+import torch
+
+from helpers import cfg_of, context, random_m, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+TOL = 2e-6
+
+
+def field(c, **kw):
+    from paper_2602_12242_gb300 import MX_TERM_DEMAG
+    from paper_2602_12242_gb300.solver import from_dev4, to_dev4
+    ctx = context(c, **kw)
+    h = from_dev4(ctx.heff(to_dev4(np.asarray(random_m(c, 41), np.float32)), terms=MX_TERM_DEMAG))
+    ctx.sync()
+    return h, ctx
+
+
+# (nx, ny, nz): Py/2 = 16 .. 512 with Pz = 4 .. 32, full and ragged nz <= Pz/2 and ny <= Py/2,
+# one and two kx columns per block (Hx above and below 608), an odd last column
+FEW_LAYERS = [(40, 9, 2), (33, 16, 16), (20, 13, 9), (64, 32, 16), (37, 21, 5), (30, 17, 13), (50, 64, 8), (40, 40, 4),
+              (41, 33, 2), (70, 128, 5), (24, 100, 4), (30, 77, 2), (20, 65, 7), (24, 256, 2), (600, 24, 2),
+              (1000, 10, 3), (513, 33, 4)]
+
+
+@pytest.mark.parametrize("shape", FEW_LAYERS)
+def test_few_layer_kernel_matches_generic_passes(shape):
+    from paper_2602_12242_gb300 import _lib
+    c = cfg_of(nx=shape[0], ny=shape[1], nz=shape[2], dx=2e-9, dy=2.5e-9, dz=3e-9)
+    h, ctx = field(c)
+    assert ctx.kernel_name("yz_fused") == "yz3_kernel"
+    ref, _ = field(c, demag_path=_lib.MX_DEMAG_GENERIC)
+    assert rel_l2(h, ref) <= TOL
