@@ -214,9 +214,9 @@ const char* mx_kernel_name(const mx_ctx* ctx, int q) {
       if (ctx->yz3) return "yz3_kernel";
       if (ctx->plane) return ctx->quad ? "yzq_kernel" : "yzh_kernel";
       return ctx->yz2d ? "yz2d_kernel" : "yz_fused_kernel";
-    case KID_Y_FWD: return "y_fwd_kernel";
-    case KID_Z_MUL: return "z_mul_kernel";
-    case KID_Y_INV: return "y_inv_kernel";
+    case KID_Y_FWD: return ctx->deep ? "deep_y_kernel" : "y_fwd_kernel";
+    case KID_Z_MUL: return ctx->deep ? "deep_z_kernel" : "z_mul_kernel";
+    case KID_Y_INV: return ctx->deep ? "deep_y_kernel" : "y_inv_kernel";
     case KID_LOCAL: return "local_kernel";
     case KID_NORMALIZE: return "normalize_kernel";
     case KID_COPY: return "copy_kernel";
@@ -291,6 +291,7 @@ mx_status mx_create(mx_ctx** out, const mx_params* p) {
   alloc((void**)&ctx->tw_m, sizeof(float2) * (g.Px > 1 ? g.Px / 2 : 1));
   alloc((void**)&ctx->tw_y, sizeof(float2) * g.Py);
   alloc((void**)&ctx->tw_yh, sizeof(float2) * (g.Py > 1 ? g.Py / 2 : 1));
+  alloc((void**)&ctx->tw_zh, sizeof(float2) * (g.Pz > 1 ? g.Pz / 2 : 1));
   alloc((void**)&ctx->tw_z, sizeof(float2) * g.Pz);
   alloc((void**)&ctx->hd, sizeof(float4) * nc);
   alloc((void**)&ctx->sa, sizeof(float4) * nc);
@@ -318,9 +319,12 @@ mx_status mx_create(mx_ctx** out, const mx_params* p) {
   std::vector<float2> tm = twiddles32(Mx);
   const int Hy = g.Py > 1 ? g.Py / 2 : 1;
   std::vector<float2> th = twiddles32(Hy);
+  const int Hz = g.Pz > 1 ? g.Pz / 2 : 1;
+  std::vector<float2> tzh = twiddles32(Hz);
   if (cudaMemcpy(ctx->tw_x, tx.data(), sizeof(float2) * g.Px, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(ctx->tw_m, tm.data(), sizeof(float2) * Mx, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(ctx->tw_yh, th.data(), sizeof(float2) * Hy, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(ctx->tw_zh, tzh.data(), sizeof(float2) * Hz, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(ctx->tw_y, ty.data(), sizeof(float2) * g.Py, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(ctx->tw_z, tz.data(), sizeof(float2) * g.Pz, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemset(ctx->flag, 0, sizeof(int)) != cudaSuccess ||
@@ -337,7 +341,7 @@ mx_status mx_destroy(mx_ctx* ctx) {
   if (!ctx) return MX_OK;
   invalidate_graph(ctx);
   adjoint_free(ctx);
-  void* ptrs[] = {ctx->ms_map, ctx->ku_map, ctx->axis_map, ctx->nhat, ctx->w1, ctx->w2, ctx->tw_x, ctx->tw_m, ctx->tw_mk, ctx->tw_yh, ctx->tw_y,
+  void* ptrs[] = {ctx->ms_map, ctx->ku_map, ctx->axis_map, ctx->nhat, ctx->w1, ctx->w2, ctx->tw_x, ctx->tw_m, ctx->tw_mk, ctx->tw_yh, ctx->tw_zh, ctx->tw_y,
                   ctx->tw_z, ctx->t_real, ctx->hd, ctx->sa, ctx->sb, ctx->acc, ctx->flag, ctx->ered, ctx->red2, ctx->dft_a, ctx->mri_f};
   for (void* q : ptrs)
     if (q) cudaFree(q);
@@ -645,7 +649,7 @@ mx_status mx_demag_spectrum(mx_ctx* ctx, float* out, mx_stream_t stream) {
     set_error("mx_demag_spectrum: demag kernel not built");
     return MX_ERR_NOT_BUILT;
   }
-  if (ctx->plane || ctx->yz3) return plane_spectrum_out(ctx, out, (cudaStream_t)stream);
+  if (ctx->octant6()) return plane_spectrum_out(ctx, out, (cudaStream_t)stream);
   const long no = (long)ctx->g.Hx * ctx->g.Oy * ctx->g.Oz;
   MX_CUDA_TRY(cudaMemcpyAsync(out, ctx->nhat, sizeof(float) * 6 * no, cudaMemcpyDeviceToDevice,
                               (cudaStream_t)stream));

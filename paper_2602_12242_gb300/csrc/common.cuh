@@ -105,7 +105,7 @@ struct Grid {
   int Hx;              // Px/2 + 1 (half spectrum along x); 1 when Px == 1
   int Oy, Oz;          // Py/2 + 1, Pz/2 + 1 (octant extents of the spectrum)
   long ncell;
-  int oct4;            // plane-path tensor octant split by qy mod 4 (else by qy mod 2)
+  int oct4;            // tensor octant layout of plane_octant_index (0, 1 or 2)
 };
 
 // Tensor octant layouts of the per-kx plane path (6 comps innermost, so one
@@ -114,18 +114,23 @@ struct Grid {
 //              of a plane (two-CTA plane kernel) each read contiguous rows;
 //   oct4 == 1: [kx][qz][qy mod 4][qy / 4][comp], Py/8 + 1 entries per class, so
 //              each CTA of the four-CTA plane kernel (one residue of ky mod 4)
-//              reads contiguous rows.
+//              reads contiguous rows;
+//   oct4 == 2: [qy][kx][qz mod 2][qz / 2][comp], so the deep-grid z kernel (one
+//              ky, one half of kz at a time) reads contiguous entries.
 __host__ __device__ __forceinline__ int plane_oct4_rows(const Grid& g) { return (g.Py >> 3) + 1; }
 __host__ __device__ __forceinline__ long plane_octant_index(const Grid& g, int kx, int comp, int qz, int qy) {
-  if (g.oct4) return ((((long)kx * g.Oz + qz) * 4 + (qy & 3)) * plane_oct4_rows(g) + (qy >> 2)) * 6 + comp;
+  if (g.oct4 == 1) return ((((long)kx * g.Oz + qz) * 4 + (qy & 3)) * plane_oct4_rows(g) + (qy >> 2)) * 6 + comp;
+  if (g.oct4 == 2) return ((((long)qy * g.Hx + kx) * 2 + (qz & 1)) * ((g.Oz + 1) >> 1) + (qz >> 1)) * 6 + comp;
   const int oyh = (g.Oy + 1) >> 1;
   return ((((long)kx * g.Oz + qz) * 2 + (qy & 1)) * oyh + (qy >> 1)) * 6 + comp;
 }
-// floats to allocate for either layout
+// floats to allocate for any of them
 __host__ __device__ __forceinline__ long plane_octant_size(const Grid& g) {
   const long two = (long)g.Hx * g.Oz * 2 * ((g.Oy + 1) >> 1) * 6;
   const long four = (long)g.Hx * g.Oz * 4 * plane_oct4_rows(g) * 6;
-  return two > four ? two : four;
+  const long deep = (long)g.Oy * g.Hx * 2 * ((g.Oz + 1) >> 1) * 6;
+  const long most = two > four ? two : four;
+  return most > deep ? most : deep;
 }
 
 struct LocalCoef {
@@ -164,7 +169,7 @@ struct mx_ctx {
 
   // demag
   bool built = false;
-  float* nhat = nullptr;          // tensor octant: [comp][qz][qy][kx], or plane_octant_index() on the plane path
+  float* nhat = nullptr;          // tensor octant: [comp][qz][qy][kx], or plane_octant_index() where octant6()
   float2* w1 = nullptr;           // 3 x nz x ny x Hx   (after the x pass)
   float2* w2 = nullptr;           // 3 x nz x Py x Hx   (after the y pass; unfused path)
   float2* tw_x = nullptr;         // W_Px^k, k < Px
@@ -173,10 +178,14 @@ struct mx_ctx {
   bool fused_yz = false;          // y/z passes in one kernel (plane fits on chip)
   bool fast_x = false;            // compile-time-sized x passes available
   bool yz3 = false;               // few-layer y/z kernel (whole kx planes in a block's shared memory) for the fused y/z pass
+  bool deep = false;              // deep-grid y and z kernels (demag_deep.cu)
   bool yz2d = false;              // single-z-plane y kernel (Pz == 1) for the fused y/z pass
   float2* tw_m = nullptr;         // W_M^k, k < M = Px/2
   float2* tw_mk = nullptr;        // W_M^(s k) at [k * S + s] for the plane path's x line FFTs (M = E S)
   float2* tw_yh = nullptr;        // W_{Py/2}^k, k < Py/2
+  float2* tw_zh = nullptr;        // W_{Pz/2}^k, k < Pz/2
+  // the octant is stored in plane_octant_index order
+  bool octant6() const { return plane || yz3 || deep; }
   bool plane = false;             // per-kx plane kernel (kx-major spectra and tensor)
   bool quad = false;              // plane path uses the four-CTA y/z kernel (else the two-CTA one)
   int xfk_grid = 1;               // persistent grid of the plane path's x forward kernel

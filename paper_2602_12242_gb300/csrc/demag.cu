@@ -321,6 +321,8 @@ mx_status demag_yz(mx_ctx* ctx, cudaStream_t st) {
   if (ctx->yz3) {
     ProfScope ps(ctx, KID_YZ, st);
     MX_TRY(yz3_pass(ctx, false, st, false));
+  } else if (ctx->deep) {
+    MX_TRY(deep_pass(ctx, st));
   } else if (ctx->yz2d) {
     ProfScope ps(ctx, KID_YZ, st);
     MX_TRY(yz2d_pass(ctx, st));

@@ -666,7 +666,8 @@ mx_status plane_setup(mx_ctx* ctx) {
   if (ctx->yz3 && !xk) ctx->fused_yz = true;
   ctx->quad = xk && !ctx->yz3 && path != MX_DEMAG_PLANE_PAIR && quad_pass(ctx, nullptr, true) == MX_OK;
   ctx->plane = ctx->quad || (xk && ctx->yz3) || (xk && yzh_pass(ctx, nullptr, true) == MX_OK);
-  ctx->g.oct4 = ctx->quad ? 1 : 0;
+  ctx->deep = path == MX_DEMAG_AUTO && ctx->fast_x && !ctx->plane && !ctx->fused_yz && deep_setup(ctx);
+  ctx->g.oct4 = ctx->quad ? 1 : (ctx->deep ? 2 : 0);
   ctx->xlocal = ctx->plane && path == MX_DEMAG_PLANE_XLOCAL;
   clear_error();
   if ((path == MX_DEMAG_PLANE || path == MX_DEMAG_PLANE_PAIR || path == MX_DEMAG_PLANE_XLOCAL) && !ctx->plane) {

@@ -48,6 +48,11 @@ mx_status fast_x_pass(mx_ctx* ctx, const float4* m, float4* hd, bool inverse, cu
 // path (setup: check the grid fits and set the kernel's attributes)
 mx_status yz3_pass(mx_ctx* ctx, bool km, cudaStream_t st, bool setup);
 
+// demag_deep.cu: the y and z passes of deep grids, w1 in place through w2
+// (deep_setup: whether the grid fits; sets the kernels' attributes)
+bool deep_setup(mx_ctx* ctx);
+mx_status deep_pass(mx_ctx* ctx, cudaStream_t st);
+
 // demag_plane.cu
 mx_status plane_setup(mx_ctx* ctx);
 mx_status plane_field(mx_ctx* ctx, const float4* m, float4* hd, cudaStream_t st);

@@ -377,7 +377,7 @@ mx_status build_demag_kernel(mx_ctx* ctx, cudaStream_t st) {
       if (status == MX_OK) {
         const long no = (long)g.Hx * g.Oy * g.Oz;
         extract_octant_kernel<<<(unsigned)((no + 255) / 256), 256, 0, st>>>(buf, c, g, ctx->nhat,
-                                                                             ctx->plane || ctx->yz3 ? 1 : 0,
+                                                                             ctx->octant6() ? 1 : 0,
                                                                              mx, mx + 1);
         status = launch_check("extract_octant_kernel");
       }

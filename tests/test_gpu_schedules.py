@@ -41,3 +41,22 @@ def test_few_layer_kernel_matches_generic_passes(shape):
     assert ctx.kernel_name("yz_fused") == "yz3_kernel"
     ref, _ = field(c, demag_path=_lib.MX_DEMAG_GENERIC)
     assert rel_l2(h, ref) <= TOL
+
+
+# (nx, ny, nz): Pz/2 = 16 .. 512 and Py/2 = 16 .. 512, full and ragged depths, a last kx tile of one
+# column (Hx = 65) and of part of one
+DEEP = [(40, 33, 64), (33, 64, 33), (20, 100, 16), (50, 20, 100), (24, 17, 129), (64, 65, 40), (17, 130, 30),
+        (16, 300, 20), (30, 12, 260), (20, 257, 17), (40, 40, 20), (100, 9, 65)]
+
+
+@pytest.mark.parametrize("shape", DEEP)
+def test_deep_grid_kernels_match_generic_passes(shape):
+    from paper_2602_12242_gb300 import _lib
+    c = cfg_of(nx=shape[0], ny=shape[1], nz=shape[2], dx=2e-9, dy=2.5e-9, dz=3e-9)
+    h, ctx = field(c)
+    assert ctx.kernel_name("z_mul") == "deep_z_kernel"
+    ref, gen = field(c, demag_path=_lib.MX_DEMAG_GENERIC)
+    assert gen.kernel_name("z_mul") == "z_mul_kernel"
+    assert rel_l2(h, ref) <= TOL
+    # the stored tensor spectrum reads back in the documented order
+    assert torch.equal(ctx.demag_spectrum(), gen.demag_spectrum())
