@@ -9,6 +9,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "xrows.cuh"
 
 namespace mx {
 
@@ -206,17 +207,17 @@ const char* mx_kernel_name(const mx_ctx* ctx, int q) {
   switch (q) {
     case KID_X_FWD:
       if (ctx->plane) return dft ? "xfk_dft_kernel" : "xfk_kernel";
-      return ctx->fast_x ? "xf_kernel" : "x_fwd_kernel";
+      return ctx->fast_x ? (few_rows(ctx->g) ? "xf_kernel" : "xf_many_kernel") : "x_fwd_kernel";
     case KID_X_INV:
       if (ctx->plane) return dft ? "xik_dft_kernel" : "xik_kernel";
-      return ctx->fast_x ? "xi_kernel" : "x_inv_kernel";
+      return ctx->fast_x ? (few_rows(ctx->g) ? "xi_kernel" : "xi_many_kernel") : "x_inv_kernel";
     case KID_YZ:
       if (ctx->yz3) return "yz3_kernel";
       if (ctx->plane) return ctx->quad ? "yzq_kernel" : "yzh_kernel";
       return ctx->yz2d ? "yz2d_kernel" : "yz_fused_kernel";
-    case KID_Y_FWD: return ctx->deep ? "deep_y_kernel" : "y_fwd_kernel";
-    case KID_Z_MUL: return ctx->deep ? "deep_z_kernel" : "z_mul_kernel";
-    case KID_Y_INV: return ctx->deep ? "deep_y_kernel" : "y_inv_kernel";
+    case KID_Y_FWD: return ctx->deep ? "deep_yf_kernel" : "y_fwd_kernel";
+    case KID_Z_MUL: return ctx->deep ? (ctx->g.Pz > 128 ? "deep_z3_kernel" : "deep_z_kernel") : "z_mul_kernel";
+    case KID_Y_INV: return ctx->deep ? "deep_yi_kernel" : "y_inv_kernel";
     case KID_LOCAL: return "local_kernel";
     case KID_NORMALIZE: return "normalize_kernel";
     case KID_COPY: return "copy_kernel";
@@ -291,7 +292,6 @@ mx_status mx_create(mx_ctx** out, const mx_params* p) {
   alloc((void**)&ctx->tw_m, sizeof(float2) * (g.Px > 1 ? g.Px / 2 : 1));
   alloc((void**)&ctx->tw_y, sizeof(float2) * g.Py);
   alloc((void**)&ctx->tw_yh, sizeof(float2) * (g.Py > 1 ? g.Py / 2 : 1));
-  alloc((void**)&ctx->tw_zh, sizeof(float2) * (g.Pz > 1 ? g.Pz / 2 : 1));
   alloc((void**)&ctx->tw_z, sizeof(float2) * g.Pz);
   alloc((void**)&ctx->hd, sizeof(float4) * nc);
   alloc((void**)&ctx->sa, sizeof(float4) * nc);
@@ -319,12 +319,9 @@ mx_status mx_create(mx_ctx** out, const mx_params* p) {
   std::vector<float2> tm = twiddles32(Mx);
   const int Hy = g.Py > 1 ? g.Py / 2 : 1;
   std::vector<float2> th = twiddles32(Hy);
-  const int Hz = g.Pz > 1 ? g.Pz / 2 : 1;
-  std::vector<float2> tzh = twiddles32(Hz);
   if (cudaMemcpy(ctx->tw_x, tx.data(), sizeof(float2) * g.Px, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(ctx->tw_m, tm.data(), sizeof(float2) * Mx, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(ctx->tw_yh, th.data(), sizeof(float2) * Hy, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(ctx->tw_zh, tzh.data(), sizeof(float2) * Hz, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(ctx->tw_y, ty.data(), sizeof(float2) * g.Py, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(ctx->tw_z, tz.data(), sizeof(float2) * g.Pz, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemset(ctx->flag, 0, sizeof(int)) != cudaSuccess ||
@@ -341,7 +338,7 @@ mx_status mx_destroy(mx_ctx* ctx) {
   if (!ctx) return MX_OK;
   invalidate_graph(ctx);
   adjoint_free(ctx);
-  void* ptrs[] = {ctx->ms_map, ctx->ku_map, ctx->axis_map, ctx->nhat, ctx->w1, ctx->w2, ctx->tw_x, ctx->tw_m, ctx->tw_mk, ctx->tw_yh, ctx->tw_zh, ctx->tw_y,
+  void* ptrs[] = {ctx->ms_map, ctx->ku_map, ctx->axis_map, ctx->nhat, ctx->w1, ctx->w2, ctx->tw_x, ctx->tw_m, ctx->tw_mk, ctx->tw_yh, ctx->tw_y,
                   ctx->tw_z, ctx->t_real, ctx->hd, ctx->sa, ctx->sb, ctx->acc, ctx->flag, ctx->ered, ctx->red2, ctx->dft_a, ctx->mri_f};
   for (void* q : ptrs)
     if (q) cudaFree(q);

@@ -115,12 +115,12 @@ struct Grid {
 //   oct4 == 1: [kx][qz][qy mod 4][qy / 4][comp], Py/8 + 1 entries per class, so
 //              each CTA of the four-CTA plane kernel (one residue of ky mod 4)
 //              reads contiguous rows;
-//   oct4 == 2: [qy][kx][qz mod 2][qz / 2][comp], so the deep-grid z kernel (one
-//              ky, one half of kz at a time) reads contiguous entries.
+//   oct4 == 2: [qy][qz][comp / 2][kx][comp mod 2], so the deep-grid z kernel (one
+//              ky, neighbouring kx on neighbouring lanes) reads contiguous pairs.
 __host__ __device__ __forceinline__ int plane_oct4_rows(const Grid& g) { return (g.Py >> 3) + 1; }
 __host__ __device__ __forceinline__ long plane_octant_index(const Grid& g, int kx, int comp, int qz, int qy) {
   if (g.oct4 == 1) return ((((long)kx * g.Oz + qz) * 4 + (qy & 3)) * plane_oct4_rows(g) + (qy >> 2)) * 6 + comp;
-  if (g.oct4 == 2) return ((((long)qy * g.Hx + kx) * 2 + (qz & 1)) * ((g.Oz + 1) >> 1) + (qz >> 1)) * 6 + comp;
+  if (g.oct4 == 2) return ((((long)qy * g.Oz + qz) * 3 + (comp >> 1)) * g.Hx + kx) * 2 + (comp & 1);
   const int oyh = (g.Oy + 1) >> 1;
   return ((((long)kx * g.Oz + qz) * 2 + (qy & 1)) * oyh + (qy >> 1)) * 6 + comp;
 }
@@ -128,9 +128,7 @@ __host__ __device__ __forceinline__ long plane_octant_index(const Grid& g, int k
 __host__ __device__ __forceinline__ long plane_octant_size(const Grid& g) {
   const long two = (long)g.Hx * g.Oz * 2 * ((g.Oy + 1) >> 1) * 6;
   const long four = (long)g.Hx * g.Oz * 4 * plane_oct4_rows(g) * 6;
-  const long deep = (long)g.Oy * g.Hx * 2 * ((g.Oz + 1) >> 1) * 6;
-  const long most = two > four ? two : four;
-  return most > deep ? most : deep;
+  return two > four ? two : four;  // (the third is the octant without padding)
 }
 
 struct LocalCoef {
@@ -183,7 +181,6 @@ struct mx_ctx {
   float2* tw_m = nullptr;         // W_M^k, k < M = Px/2
   float2* tw_mk = nullptr;        // W_M^(s k) at [k * S + s] for the plane path's x line FFTs (M = E S)
   float2* tw_yh = nullptr;        // W_{Py/2}^k, k < Py/2
-  float2* tw_zh = nullptr;        // W_{Pz/2}^k, k < Pz/2
   // the octant is stored in plane_octant_index order
   bool octant6() const { return plane || yz3 || deep; }
   bool plane = false;             // per-kx plane kernel (kx-major spectra and tensor)

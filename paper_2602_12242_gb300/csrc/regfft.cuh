@@ -128,6 +128,23 @@ template <int E, int S> struct LineFft {
   static constexpr int kPitch = (S > 1) ? E * (S + 1) : E;
 };
 
+// Shared-memory line layout.  A half-warp of a line FFT covers H = 16 / S
+// lines, and load and store loops may put T neighbouring lines on neighbouring
+// lanes.  Both stay free of bank conflicts when the H lines of a group start
+// 2 S words apart modulo 32 and the groups 4 words apart.
+template <int E, int S> struct BankLine {
+  static constexpr int PITCH = LineFft<E, S>::kPitch;
+  static constexpr int H = S >= 16 ? 1 : 16 / S;
+  // shift of lines within a group (a multiple of 2 S words apart), and the group's stride
+  static constexpr bool SHIFT = (S == 8 && PITCH % 16 == 0) || (S == 4 && PITCH % 16 == 8);
+  static constexpr int GROUP = H * PITCH + (SHIFT ? 16 : 0) + 2;
+  __device__ __forceinline__ static int off(int l) {
+    const int r = l % H;
+    return l / H * GROUP + r * PITCH + (SHIFT ? (S == 8 ? 8 * r : 4 * (r >> 1)) : 0);
+  }
+  static constexpr int size(int lines) { return (lines + H - 1) / H * GROUP; }  // float2 of `lines` lines
+};
+
 // Second step of line_fft: the twiddled E x S matrix is in rows k1 * (S + 1);
 // thread s does S-point FFTs over s for k1 = s + S j and writes X[k1 + E k2]
 // in natural order.

@@ -213,8 +213,8 @@ template <class F> mx_status few_rows_dispatch(int half, F& f) {
     case 256: return f.template run<16, 16, 1, few_rows_nt<16, 1>()>();
     case 128: return f.template run<16, 8, 1, few_rows_nt<8, 1>()>();
     case 64: return f.template run<8, 8, 2, few_rows_nt<8, 2>()>();
-    case 32: return f.template run<32, 1, 4, few_rows_nt<1, 4>()>();
-    case 16: return f.template run<16, 1, 4, few_rows_nt<1, 4>()>();
+    case 32: return f.template run<8, 4, 4, few_rows_nt<4, 4>()>();
+    case 16: return f.template run<4, 4, 4, few_rows_nt<4, 4>()>();
     default: return MX_ERR_UNSUPPORTED;
   }
 }

@@ -54,9 +54,27 @@ def test_deep_grid_kernels_match_generic_passes(shape):
     from paper_2602_12242_gb300 import _lib
     c = cfg_of(nx=shape[0], ny=shape[1], nz=shape[2], dx=2e-9, dy=2.5e-9, dz=3e-9)
     h, ctx = field(c)
-    assert ctx.kernel_name("z_mul") == "deep_z_kernel"
+    assert ctx.kernel_name("z_mul") == ("deep_z3_kernel" if ctx.padded_dims[2] > 128 else "deep_z_kernel")
     ref, gen = field(c, demag_path=_lib.MX_DEMAG_GENERIC)
     assert gen.kernel_name("z_mul") == "z_mul_kernel"
     assert rel_l2(h, ref) <= TOL
     # the stored tensor spectrum reads back in the documented order
     assert torch.equal(ctx.demag_spectrum(), gen.demag_spectrum())
+
+
+# (nx, ny, nz) with many rows: every row length Px/2 = 16 .. 1024 of the many-row x kernels, odd nx,
+# a last block of part of its rows
+ROWS = [(9, 101, 99), (17, 100, 101), (33, 70, 60), (127, 61, 43), (129, 41, 33), (300, 37, 35), (520, 33, 31)]
+
+
+@pytest.mark.parametrize("shape", ROWS)
+@pytest.mark.parametrize("ms_map", [False, True])
+def test_many_row_x_kernels_match_generic_passes(shape, ms_map):
+    from paper_2602_12242_gb300 import _lib
+    c = cfg_of(nx=shape[0], ny=shape[1], nz=shape[2], dx=2e-9, dy=2.5e-9, dz=3e-9)
+    Ms = np.random.default_rng(43).uniform(6e5, 1e6, size=shape[::-1]) if ms_map else None
+    h, ctx = field(c, Ms=Ms)
+    assert (ctx.kernel_name("x_fwd"), ctx.kernel_name("x_inv")) == ("xf_many_kernel", "xi_many_kernel")
+    ref, gen = field(c, Ms=Ms, demag_path=_lib.MX_DEMAG_GENERIC)
+    assert gen.kernel_name("x_fwd") == "x_fwd_kernel"
+    assert rel_l2(h, ref) <= TOL
