@@ -188,3 +188,39 @@ def test_training_reduces_loss_and_in_loop_fallback():
     m2 = M[1].clone()
     res2 = run_in_loop(ctx, net, m2, nsteps=6, dt=1e-14, judge_every=3, threshold=10.0)
     assert res2["fallback_step"] is None and len(res2["errors"]) == 2
+
+
+@pytest.mark.parametrize("nx,ny,K,B", [(8, 40, 3, 1), (41, 32, 16, 4), (41, 32, 16, 6), (166, 20, 9, 9), (1022, 16, 8, 2),
+                                       (20, 200, 10, 5), (64, 24, 1, 7)])
+def test_launch_variants_match_oracle(nx, ny, K, B):
+    """Both sides of each launch rule (rows per SM, samples per batch, rows too long for
+    staged twiddles) at odd widths, mode counts that are no multiple of four or eight, a
+    number of rows of less than an eighth of the cluster's share: outputs and gradients
+    against the oracle, at the tolerances of the tests above."""
+    flat = params_for(K, 21)
+    m = fields(B, ny, nx, 22)
+    net = make_net(nx, ny, K, B, flat)
+    h = net.forward(dev4(m))[..., :3].double().cpu().numpy().reshape(oracle_h(flat, m, K).shape)
+    assert rel_l2(h, oracle_h(flat, m, K)) <= 2e-5
+    ht = fields(B, ny, nx, 23) * 3e4
+    loss, grad = net.loss_grad(dev4(m), dev4(ht))
+    x = fno.to_nchw((m - STATS[0:3]) / STATS[3:6])
+    t = fno.to_nchw((ht - STATS[6:9]) / STATS[9:12])
+    L, ref = fno.loss_and_grad(torch.from_numpy(flat), x, t, K)
+    assert abs(float(loss) - L) <= 1e-5 * abs(L)
+    g, ref = grad.double().cpu().numpy(), ref.numpy()
+    offs = np.cumsum([0] + [int(np.prod(s)) for s in fno.param_shapes(K)])
+    for i in range(len(offs) - 1):
+        assert rel_l2(g[offs[i]:offs[i + 1]], ref[offs[i]:offs[i + 1]]) <= 1e-4, i
+
+
+@pytest.mark.parametrize("nx,ny,K", [(160, 40, 12), (41, 70, 5), (37, 20, 9)])
+def test_output_does_not_depend_on_the_batch_size(nx, ny, K):
+    """The launch variants sum in one order: a sample alone, in a small batch and in a large
+    one has the same output bit for bit."""
+    flat = params_for(K, 31)
+    m = fields(12, ny, nx, 32)
+    net = make_net(nx, ny, K, 12, flat)
+    full = net.forward(dev4(m)).cpu()
+    for b in (1, 2, 4, 5, 8):
+        assert torch.equal(net.forward(dev4(m[3:3 + b])).cpu(), full[3:3 + b]), b
