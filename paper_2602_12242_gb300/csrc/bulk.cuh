@@ -45,6 +45,18 @@ __device__ __forceinline__ void bulk_load(void* dst_smem, const void* src, uint3
                : "memory");
 }
 
+// A box of a 3D tensor map, innermost coordinate x in elements (a multiple of 16
+// bytes), into shared memory (128-byte aligned); completes its bytes on `bar`.
+// A copy of many short rows is one instruction this way: separate bulk_load
+// copies of 160 to 256 bytes go out at one per 40 ns and SM.
+__device__ __forceinline__ void tensor_load3(void* dst_smem, const void* map, int x, int y, int z, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
+          smem_u32addr(dst_smem)),
+      "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32addr(bar))
+      : "memory");
+}
+
 // shared -> global, in the issuing thread's current bulk group
 __device__ __forceinline__ void bulk_store(void* dst, const void* src_smem, uint32_t bytes) {
   asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32addr(src_smem)),
@@ -71,12 +83,19 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 
 // Bounded wait for the completion of phase `parity` of `bar`: false after
-// about kBulkWaitNs of global time (checked every 256 polls).
+// about kBulkWaitNs of global time (checked every 256 polls, and first read
+// then: the timer's read takes longer than a short wait).
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   const uint32_t a = smem_u32addr(bar);
-  const unsigned long long t0 = global_ns();
+  unsigned long long t0 = 0;
   for (int i = 0; i < kBulkWaitPolls; ++i) {
-    if ((i & 255) == 255 && global_ns() - t0 > kBulkWaitNs) return false;
+    if ((i & 255) == 255) {
+      const unsigned long long t = global_ns();
+      if (t0 == 0)
+        t0 = t;
+      else if (t - t0 > kBulkWaitNs)
+        return false;
+    }
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"

@@ -5,20 +5,24 @@
 // Sec. II-D: a network trained offline on (M, H_demag) pairs from the FFT
 // solver, per-channel Gaussian normaliser, Adam lr 1e-3, weight decay 1e-4).
 //
-// Activations are BF16, channels-last [b][z][y][x][C] with C padded to a
-// multiple of 16 (first input: 3 -> 16); weights are FP32 masters with BF16
-// copies for the tensor cores.  Every convolution is an implicit GEMM on the
-// tcgen05 tensor cores (BF16 in, FP32 accumulator in tensor memory): a block
-// takes 8 x 16 x 1 tiles of output cells (M = 128) with a (10 x 18 x 3) halo
-// of input cells staged with cp.async; all 27 taps of the layer's weights
-// stay in shared memory.  The weight gradient runs on tcgen05 too, with
-// MN-major operands (wgrad_tc_kernel).
+// Activations are BF16 planes of eight channels, [b z][C/8][y][x][8] with C
+// padded to a multiple of 16 (first input: 3 -> 16), and a border of zero cells
+// around every plane (x, y = -1 and up to the tile grid's end) that is written
+// once, at creation.  So every operand tile, halo included, is a set of
+// contiguous rows that bulk copies fetch without a bounds check, and each
+// thread of an epilogue stores 16 bytes next to its neighbour's.  Weights are
+// FP32 masters with BF16 copies in the layout of the tensor cores' operand.
 //   forward     out = conv(a, W) + b, stored pre-activation y and a = gelu(y)
 //   backward-x  dA_{l-1} = conv(dY_l, W'), W'[tap][ci][co] = W[26 - tap][co][ci],
 //               times gelu'(y_{l-1}) in the epilogue -> dY_{l-1}
-//   backward-W  dW[tap] = sum over cells of dY (x) x_shifted(tap), one block per
-//               (dz, ddy, chunk of tiles) with its three taps in tensor memory,
-//               FP32 atomics into the gradient
+//   backward-W  dW[tap] = sum over cells of dY (x) x_shifted(tap)
+// Every convolution and weight gradient is a tcgen05 (BF16 in, FP32 accumulator
+// in tensor memory) kernel of three roles: a producer warp issues the bulk
+// copies, one thread the MMAs, eight warps run the epilogue of the tile before;
+// they meet at mbarriers only (every wait bounded; one that runs out sets
+// kFlagTimeout and its role stops).  The last layer's epilogue denormalises, or
+// in training forms the loss and its gradient.
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <math.h>
 #include <string.h>
@@ -34,453 +38,545 @@
 
 namespace mx {
 
-constexpr int kTX = 16, kTY = 8;             // output tile (cells)
-constexpr int kHX = kTX + 2, kHY = kTY + 2;  // halo
-constexpr int kHalo = kHX * kHY * 3;
-constexpr int kCnnThreads = 256;
 static const int kCh[5] = {3, 32, 64, 32, 3};
 static const int kCinPad[4] = {16, 32, 64, 32};
-static const int kCoutPad[4] = {32, 64, 32, 8};
+static const int kCoutPad[4] = {32, 64, 32, 16};
 
 __device__ __forceinline__ float gelu_f(float y) { return 0.5f * y * (1.f + erff(y * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_grad(float y) {
   return 0.5f * (1.f + erff(y * 0.70710678118654752f)) + y * 0.39894228040143268f * expf(-0.5f * y * y);
 }
 
+// Grid and storage of one activation: rows of wq cells, planes of hp rows.
 struct ConvDims {
   int nx, ny, nz, batch;
-  int tiles_x, tiles_y, ntiles;  // tiles per (b, z) plane and total
+  int wq, hp;
+};
+// cells from the start of a stored plane to cell (x, y)
+__device__ __forceinline__ long cell_at(const ConvDims& d, int y, int x) { return (long)(y + 1) * d.wq + x + 1; }
+
+// A CTA's tiles [t0, t1): tile t is layer z = t % nz of column t / nz.  The
+// planes z - 1 .. z + 1 inside the grid are loaded once per column (or at the
+// range's start) into a ring of slots, in order.  A tile holds at most three; the
+// slots beyond them are what the producer can run ahead, and a copy's latency is
+// about that of a tile's MMAs.
+struct TileWalk {
+  int t0, t1, nz;
+  __device__ TileWalk(long ntiles, int cta, int ncta, int nz_) : nz(nz_) {
+    t0 = (int)(ntiles * cta / ncta);
+    t1 = (int)(ntiles * (cta + 1) / ncta);
+  }
+  // planes of tile t that are not loaded yet: [z0, z1]
+  __device__ void fresh(int t, int& z0, int& z1) const {
+    const int z = t % nz;
+    z1 = min(nz - 1, z + 1);
+    z0 = (t == t0 || z == 0) ? max(0, z - 1) : z + 1;
+  }
 };
 
-__host__ __device__ inline void tile_coords(const ConvDims& d, int t, int& b, int& z, int& y0, int& x0) {
-  const int tx = t % d.tiles_x;
-  int r = t / d.tiles_x;
-  const int ty = r % d.tiles_y;
-  r /= d.tiles_y;
-  z = r % d.nz;
-  b = r / d.nz;
-  y0 = ty * kTY;
-  x0 = tx * kTX;
+// Bounded barrier wait of a role: false (and kFlagTimeout set) when it runs out.
+__device__ __forceinline__ bool role_wait(uint64_t* bar, uint32_t parity, int* flag) {
+  if (mbar_wait(bar, parity)) return true;
+  atomicOr(flag, kFlagTimeout);
+  return false;
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32addr(bar)) : "memory");
 }
 
-enum ConvMode { CM_HIDDEN = 0, CM_LAST = 1, CM_BWD = 2 };
+enum ConvMode { CM_HIDDEN = 0, CM_BWD = 1, CM_OUT = 2, CM_LOSS = 3 };
+
+struct ConvArgs {
+  const bf16_t* wk;    // [27][CIN/8][NP][8]
+  const float* bias;
+  bf16_t* out;         // HIDDEN: gelu; BWD: dY of the layer below; LOSS: dY of the last layer (channels 0..7)
+  bf16_t* ypre;        // HIDDEN: pre-activation (may be null); BWD: read
+  const float4* target;  // LOSS: raw target field
+  float4* field;       // OUT: denormalised field
+  float* db;           // BWD, LOSS: bias gradient of the layer whose dY is written
+  float* loss;         // LOSS
+  float3 mean, sd;     // OUT: of the field; LOSS: mean and 1 / std
+  float inv_count;     // LOSS
+  ConvDims d;
+  int* flag;
+};
 
 // ---------------------------------------------------------------------------
-// Convolution: in [cells][CIN] (bf16), weights wk [27][COUT][CIN] (bf16), on
-// the tcgen05 tensor cores, one persistent block per SM looping over tiles.
-//   CM_HIDDEN: ypre = acc + b (bf16), out = gelu(acc + b) (bf16), [cells][COUT]
-//   CM_LAST:   outf = acc + b (fp32) channels 0..2 of a float4 record per cell
-//   CM_BWD:    out = acc * gelu'(ypre) (bf16), [cells][COUT]  (ypre read)  A block (persistent, one
-// per SM) takes an 8 (x) x 16 (y) x 1 tile of output cells, M = 128 rows
-// (row = 8 y + x); N = COUT (16 for the last layer, whose padding rows are
-// zero weights); K = 27 taps x CIN.  Shared memory holds every operand in the
-// canonical K-major layout without swizzle:
+// Convolution as an implicit GEMM.  A tile is 8 (x) x 16 (y) x 1 output cells, M =
+// 128 rows (row = 8 y + x); N = COUT (16 for the last layer); K = 27 taps x CIN.
+// Operands in the canonical K-major layout without swizzle:
 //   weights [tap][CIN/8][N][8]   B of tap t, K chunk c: 8-row groups (8 output
 //                                channels) 128 B apart, K chunks N x 16 B apart
-//   halo    [CIN/8][540][8]      (3 x 18 x 10 cells): A of tap (dz, dy, dx) starts
-//                                at cell (dz, dy, dx); consecutive x are 16 B
-//                                apart, so each output row y (8 cells) is one
-//                                8-row group and groups are 10 x 16 B apart
-// One thread issues the 27 CIN/16 MMAs of a tile into a TMEM accumulator
-// (128 lanes x N columns, FP32) and commits them to an mbarrier; after the
-// (bounded) wait, warp w reads lanes 32 (w mod 4) .. +31, columns of half
-// w / 4, for the epilogue.
+//   plane   [CIN/8][180][8]      (18 x 10 cells): A of tap (dz, dy, dx) starts at
+//                                cell (dy, dx) of plane z + dz - 1; each output
+//                                row y (8 cells) is one 8-row group, groups are
+//                                10 x 16 B apart
+// Taps of a plane outside the grid are left out (their products are zero).  A
+// CTA walks z fastest, so each tile brings one new plane; the planes of tile t +
+// 1 arrive and its MMAs start while the epilogue of tile t runs (two accumulators
+// in tensor memory).
+// Bound: the MMAs, at 60 to 80 cycles each whatever N <= 64 is (their A operand is 4
+// KB of shared memory), and for 64 output channels the issue slots of the epilogue's
+// erf.  Measured forward at 64 samples of 64x64x4, with the kernel before in brackets
+// (256 threads copied three planes per tile with cp.async, waited for the MMAs and
+// ran the epilogue in turn): 3 -> 32 channels 98 us (230), 32 -> 64 167 (362), 64 ->
+// 32 191 (475), 32 -> 3 with the loss 104 (268 + 51).  On the way: planes as separate
+// bulk copies of their 160-byte rows went out at one per 40 ns (64 -> 32 290 us); a
+// single diverged thread issuing the MMAs took 20 cycles more for each than a
+// converged warp with uniform operands; column coordinates divided out per tile cost
+// 5 %.
 // ---------------------------------------------------------------------------
 constexpr int kTXc = 8, kTYc = 16;
 constexpr int kHXc = kTXc + 2, kHYc = kTYc + 2;
-constexpr int kHaloC = kHXc * kHYc * 3;
+constexpr int kPlaneC = kHXc * kHYc;
 
 template <int CIN, int COUT> struct ConvTc {
   static constexpr int NP = COUT < 16 ? 16 : COUT;  // MMA N
   static constexpr int KC = CIN / 8;
-  static constexpr size_t w_bytes = sizeof(bf16_t) * 8 * 27 * KC * NP;
-  static constexpr size_t h_bytes = sizeof(bf16_t) * 8 * KC * kHaloC;
-  // two halo buffers where they fit next to the weights (227 KB)
-  static constexpr int NB = (w_bytes + 2 * h_bytes <= 227 * 1024) ? 2 : 1;
-  static constexpr size_t smem = w_bytes + NB * h_bytes;
+  static constexpr int EW = COUT < 16 ? 8 : 16;     // epilogue warps: four lane quarters x EW / 4 column parts
+  static constexpr int threads = 32 * (2 + EW);
+  static constexpr uint32_t w_bytes = sizeof(bf16_t) * 8 * 27 * KC * NP;
+  static constexpr uint32_t p_bytes = sizeof(bf16_t) * 8 * KC * kPlaneC;
+  // as many plane slots as fit, at most 8 (at least 4)
+  static constexpr int FIT = (int)((226 * 1024 - w_bytes) / p_bytes);
+  static constexpr int RING = FIT < 8 ? FIT : 8;
+  static_assert(RING >= 4, "three planes of a tile and one to load");
+  static constexpr size_t smem = w_bytes + RING * p_bytes;
   // two accumulators of NP columns, allocated as a power of two >= 32
-  static constexpr uint32_t TCOLS = 2 * NP <= 32 ? 32 : (2 * NP <= 64 ? 64 : (2 * NP <= 128 ? 128 : 256));
+  static constexpr uint32_t TCOLS = 2 * NP <= 32 ? 32 : (2 * NP <= 64 ? 64 : 128);
 };
 
 template <int CIN, int COUT, int MODE>
-__global__ void __launch_bounds__(kCnnThreads, 1) conv_tc_kernel(const bf16_t* __restrict__ in,
-                                                                  const bf16_t* __restrict__ wk,
-                                                                  const float* __restrict__ bias,
-                                                                  bf16_t* __restrict__ out, bf16_t* __restrict__ ypre,
-                                                                  float4* __restrict__ outf, ConvDims d, int* flag) {
+__global__ void __launch_bounds__(ConvTc<CIN, COUT>::threads, 1)
+    conv_tc_kernel(const __grid_constant__ CUtensorMap in, const __grid_constant__ ConvArgs p) {
   typedef ConvTc<CIN, COUT> T;
-  constexpr int NP = T::NP, KC = T::KC, NH = NP / 2, NB = T::NB;
-  const int cta = (int)blockIdx.x, ncta = (int)gridDim.x;
+  constexpr int RING = T::RING, NP = T::NP, KC = T::KC, NH = NP / (T::EW / 4);
   extern __shared__ __align__(128) unsigned char smraw[];
-  __shared__ __align__(8) uint64_t bar[2];
+  __shared__ __align__(8) uint64_t wbar, full[RING], empty[RING], tfull[2], tempty[2];
   __shared__ uint32_t tbase;
-  bf16_t* sw = (bf16_t*)smraw;  // [27][KC][NP][8]
+  const ConvDims& d = p.d;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int e = tid; e < 27 * KC * NP; e += kCnnThreads) {
-    const int co = e % NP, kc = (e / NP) % KC, tap = e / (NP * KC);
-    const bool ok = co < COUT;
-    cp_async16(smem_u32(sw + (long)e * 8), wk + ((long)tap * COUT + (ok ? co : 0)) * CIN + kc * 8, ok);
-  }
-  if (warp == 0) tmem_alloc(&tbase, T::TCOLS);
+  const uint32_t sw_a = smem_u32(smraw), sp_a = sw_a + T::w_bytes;
   if (tid == 0) {
-    mbar_init(&bar[0], 1);
-    mbar_init(&bar[1], 1);
+    mbar_init(&wbar, 1);
+    for (int q = 0; q < RING; ++q) {
+      mbar_init(&full[q], 1);
+      mbar_init(&empty[q], 1);
+    }
+    for (int q = 0; q < 2; ++q) {
+      mbar_init(&tfull[q], 1);
+      mbar_init(&tempty[q], T::EW);
+    }
   }
-  const uint32_t sw_a = smem_u32(sw);
-  const uint32_t sh_a0 = sw_a + (uint32_t)T::w_bytes;
-  constexpr uint32_t idesc = tc_idesc_bf16(128, NP);
-  const int tiles_x = (d.nx + kTXc - 1) / kTXc, tiles_y = (d.ny + kTYc - 1) / kTYc;
-  const int ntiles = tiles_x * tiles_y * d.nz * d.batch;
-  const int nmine = cta < ntiles ? (ntiles - 1 - cta) / ncta + 1 : 0;
-  const long plane = (long)d.nx * d.ny;
-  // this thread's accumulator row: cell (cx, cy) of the tile; lane quarter, column half
-  const int row = 32 * (warp & 3) + lane;
-  const int cx = row & 7, cy = row >> 3;
-  const int cb = (warp >> 2) * NH;
-  auto coords = [&](int k, int& b, int& z, int& y0, int& x0) {
-    const int t = cta + k * ncta;
-    const int tx = t % tiles_x;
-    int r = t / tiles_x;
-    const int ty = r % tiles_y;
-    r /= tiles_y;
-    z = r % d.nz;
-    b = r / d.nz;
-    x0 = tx * kTXc;
-    y0 = ty * kTYc;
-  };
-  // halo of tile k into buffer k % NB: issue the cp.async copies as one group
-  // (halo_ready waits for them and makes them visible to the tensor core)
-  auto load_halo = [&](int k) {
-    int b, z, y0, x0;
-    coords(k, b, z, y0, x0);
-    bf16_t* sh = (bf16_t*)(smraw + T::w_bytes + (k % NB) * T::h_bytes);
-    for (int e = tid; e < kHaloC * KC; e += kCnnThreads) {
-      const int hc = e % kHaloC, kc = e / kHaloC;
-      const int hx = hc % kHXc, hy = (hc / kHXc) % kHYc, hz = hc / (kHXc * kHYc);
-      const int gx = x0 + hx - 1, gy = y0 + hy - 1, gz = z + hz - 1;
-      const bool ok = gx >= 0 && gx < d.nx && gy >= 0 && gy < d.ny && gz >= 0 && gz < d.nz;
-      const long cell = ok ? ((long)b * d.nz + gz) * plane + (long)gy * d.nx + gx : 0;
-      cp_async16(smem_u32(sh + (long)e * 8), in + cell * CIN + kc * 8, ok);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  auto halo_ready = [&]() {
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    fence_proxy_async_smem();
-  };
-  // the 27 CIN/16 MMAs of tile k into accumulator k & 1 (one thread)
-  auto issue = [&](int k) {
-    const uint32_t sh_a = sh_a0 + (uint32_t)((k % NB) * T::h_bytes);
-    const uint32_t dt = tbase + (uint32_t)((k & 1) * NP);
-    tc_fence_after_sync();
-#pragma unroll 1
-    for (int tap = 0; tap < 27; ++tap) {
-      const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
-      const uint32_t aoff = (uint32_t)(((dz * kHYc + dy) * kHXc + dx) * 16);
-#pragma unroll
-      for (int ks = 0; ks < CIN / 16; ++ks) {
-        const uint64_t ad = tc_sdesc(sh_a + (uint32_t)(2 * ks * kHaloC * 16) + aoff, kHaloC * 16, kHXc * 16);
-        const uint64_t bd = tc_sdesc(sw_a + (uint32_t)((tap * KC + 2 * ks) * NP * 16), NP * 16, 128);
-        tc_mma_bf16(dt, ad, bd, idesc, tap > 0 || ks > 0);
-      }
-    }
-    tc_commit(&bar[k & 1]);
-  };
-  uint32_t par[2] = {0u, 0u};
-  auto wait_mma = [&](int k) {
-    if (!mbar_wait(&bar[k & 1], par[k & 1])) atomicOr(flag, kFlagTimeout);
-    par[k & 1] ^= 1u;
-    tc_fence_after_sync();
-  };
-  cp_async_wait_all();  // weights
-  if (nmine > 0) {
-    load_halo(0);
-    halo_ready();
-  }
-  tc_fence_before_sync();
-  __syncthreads();
-  if (nmine > 0 && tid == 0) issue(0);
-  if (NB == 2 && nmine > 1) load_halo(1);  // buffer 1 is free: prefetch
-  for (int k = 0; k < nmine; ++k) {
-    if (NB == 2) {
-      if (k + 1 < nmine) {
-        halo_ready();  // tile k + 1's halo (prefetched) is in buffer (k + 1) % 2
-        tc_fence_before_sync();
-        __syncthreads();
-        if (tid == 0) issue(k + 1);
-      }
-      wait_mma(k);  // buffer k % 2 and accumulator k & 1 are done with
-      if (k + 2 < nmine) load_halo(k + 2);  // lands during the epilogue
-    } else {
-      wait_mma(k);  // the only halo buffer is free once tile k's MMAs are done
-      if (k + 1 < nmine) {
-        load_halo(k + 1);
-        halo_ready();
-        tc_fence_before_sync();
-        __syncthreads();
-        if (tid == 0) issue(k + 1);
-      }
-    }
-    // epilogue of tile k (overlaps the MMAs of tile k + 1)
-    float v[NH];
-#pragma unroll
-    for (int q = 0; q < NH / 8; ++q) {
-      float t8[8];
-      tmem_ld8(tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((k & 1) * NP + cb + 8 * q), t8);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) v[8 * q + i] = t8[i];
-    }
-    int b, z, y0, x0;
-    coords(k, b, z, y0, x0);
-    const int gx = x0 + cx, gy = y0 + cy;
-    if (gx < d.nx && gy < d.ny) {
-      const long cell = ((long)b * d.nz + z) * plane + (long)gy * d.nx + gx;
-      // eight channels per 16-byte store
-#pragma unroll
-      for (int c = 0; c < NH; c += 8) {
-        const int cg = cb + c;  // channel of v[c]
-        if (cg >= COUT) break;
-        if (MODE == CM_HIDDEN) {
-          uint32_t yp[4], o[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float v0 = v[c + 2 * j] + bias[cg + 2 * j], v1 = v[c + 2 * j + 1] + bias[cg + 2 * j + 1];
-            yp[j] = pack2(v0, v1);
-            o[j] = pack2(gelu_f(v0), gelu_f(v1));
-          }
-          *(uint4*)(ypre + cell * COUT + cg) = make_uint4(yp[0], yp[1], yp[2], yp[3]);
-          *(uint4*)(out + cell * COUT + cg) = make_uint4(o[0], o[1], o[2], o[3]);
-        } else if (MODE == CM_BWD) {
-          const uint4 y4 = *(const uint4*)(ypre + cell * COUT + cg);
-          const uint32_t yw[4] = {y4.x, y4.y, y4.z, y4.w};
-          uint32_t o[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float y0f = bf2f((bf16_t)(yw[j] & 0xffff)), y1f = bf2f((bf16_t)(yw[j] >> 16));
-            o[j] = pack2(v[c + 2 * j] * gelu_grad(y0f), v[c + 2 * j + 1] * gelu_grad(y1f));
-          }
-          *(uint4*)(out + cell * COUT + cg) = make_uint4(o[0], o[1], o[2], o[3]);
-        } else {
-          float* o = (float*)(outf + cell);
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            if (cg + j < 3) o[cg + j] = v[c + j] + bias[cg + j];
-        }
-      }
-    }
-    tc_fence_before_sync();
-    __syncthreads();  // accumulator k & 1 and halo buffer k % NB may be reused
-  }
-  if (warp == 0) {
-    tc_fence_after_sync();
-    tmem_dealloc(tbase, T::TCOLS);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Weight gradient of one layer on the tcgen05 tensor cores:
-//   dW[tap][co][ci] += sum_cells dY[cell][co] * x[cell + off(tap)][ci].
-// Block (range of 16 x 8 output tiles, dz, ddy) owns the three taps
-// (dz, ddy, ddx = 0..2).  Per tile and tile row cy, three MMAs
-// D_ddx (co x ci) += dY^T (co x the 16 cells of row cy) X_ddx (those cells
-// shifted by the tap x ci), M = 128 (co, rows >= COUT zero), N = CIN, K = 16,
-// accumulated in tensor memory over all of the block's tiles.  Both operands
-// are MN-major (channels contiguous, one 16-byte row of 8 channels per cell,
-// core matrices adjacent along K 128 B apart, 8-channel groups SBO apart), so
-// they are 16-byte copies of the [cell][channel] activations: dY of the tile
-// (row q = cell cy * 16 + cx) and the tile's band of x rows for this ddy
-// (8 rows of 18 cells, row r * 18 + hx); the operand of (cy, ddx) starts at
-// row cy * 16 of dY and row cy * 18 + ddx of the band.
-// ---------------------------------------------------------------------------
-template <int CIN, int COUT> struct WgradShape {
-  static constexpr int HXp = kTX + 2;                    // band row: 18 cells
-  static constexpr int NROW = kTY * HXp;                 // 144 band cells
-  static constexpr uint32_t A_SBO = kTX * kTY * 16 + 16;  // 128 cells + 16 B pad (bank spread)
-  static constexpr uint32_t B_SBO = NROW * 16 + 16;
-  static constexpr uint32_t A_BYTES = 16 * A_SBO;
-  static constexpr uint32_t BUF = A_BYTES + (CIN / 8) * B_SBO;  // one tile's operands
-  static constexpr size_t smem = BUF;
-  static constexpr int TCOLS = 3 * CIN <= 64 ? 64 : (3 * CIN <= 128 ? 128 : 256);
-};
-
-template <int CIN, int COUT>
-__global__ void __launch_bounds__(kCnnThreads, 1) wgrad_tc_kernel(const bf16_t* __restrict__ x,
-                                                                  const bf16_t* __restrict__ dy,
-                                                                  float* __restrict__ dw, ConvDims d, int cin_real,
-                                                                  int cout_real, int tiles_per_block, int* flag) {
-  typedef WgradShape<CIN, COUT> W;
-  static_assert(COUT % 8 == 0 && COUT <= 128 && CIN % 16 == 0 && 3 * CIN <= 256, "wgrad shape");
-  extern __shared__ __align__(128) unsigned char smraw[];
-  __shared__ uint64_t bar;
-  __shared__ uint32_t tbase;
-  const int dz = blockIdx.y / 3, ddy = blockIdx.y % 3;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // dY^T (16 channel groups, those >= COUT/8 stay zero) then the x band
-  for (int i = tid; i < (int)(W::smem / 16); i += kCnnThreads) ((uint4*)smraw)[i] = make_uint4(0u, 0u, 0u, 0u);
-  if (warp == 0) tmem_alloc(&tbase, W::TCOLS);
-  if (tid == 0) mbar_init(&bar, 1);
+  if (warp == 1) tmem_alloc(&tbase, T::TCOLS);
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tb = tbase;
-  const long plane = (long)d.nx * d.ny;
-  const int t0 = blockIdx.x * tiles_per_block;
-  const int n = max(0, min(d.ntiles, t0 + tiles_per_block) - t0);
-  constexpr uint32_t idesc = tc_idesc_bf16(128, CIN) | (1u << 15) | (1u << 16);  // A and B MN-major
-  // the copies of tile k, as one cp.async group
-  auto stage = [&](int k) {
-    unsigned char* sA = smraw;
-    unsigned char* sB = sA + W::A_BYTES;
-    int b, z, y0, x0;
-    tile_coords(d, t0 + k, b, z, y0, x0);
-    const int gz = z + dz - 1;
-    // band cell (r, hx) -> x cell (gz, y0 + r + ddy - 1, x0 + hx - 1); chunk fastest (coalesced reads)
-    for (int e = tid; e < W::NROW * (CIN / 8); e += kCnnThreads) {
-      const int ch = e % (CIN / 8), c = e / (CIN / 8);
-      const int gx = x0 + c % W::HXp - 1, gy = y0 + c / W::HXp + ddy - 1;
-      const bool ok = gx >= 0 && gx < d.nx && gy >= 0 && gy < d.ny && gz >= 0 && gz < d.nz;
-      const long cell = ok ? ((long)b * d.nz + gz) * plane + (long)gy * d.nx + gx : 0;
-      cp_async16(smem_u32(sB + ch * W::B_SBO + c * 16), x + cell * CIN + ch * 8, ok);
-    }
-    // dY of the tile's output cells (zero outside the grid, so those cells add nothing)
-    for (int e = tid; e < kTX * kTY * (COUT / 8); e += kCnnThreads) {
-      const int ch = e % (COUT / 8), q = e / (COUT / 8);
-      const int ox = x0 + q % kTX, oy = y0 + q / kTX;
-      const bool ok = ox < d.nx && oy < d.ny;
-      const long cell = ok ? ((long)b * d.nz + z) * plane + (long)oy * d.nx + ox : 0;
-      cp_async16(smem_u32(sA + ch * W::A_SBO + q * 16), dy + cell * COUT + ch * 8, ok);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
+  const int tiles_x = (d.nx + kTXc - 1) / kTXc, tiles_y = (d.ny + kTYc - 1) / kTYc;
+  const TileWalk walk((long)tiles_x * tiles_y * d.nz * d.batch, blockIdx.x, gridDim.x, d.nz);
+  // column col: first cell of its tile, sample
+  auto column = [&](int col, int& b, int& y0, int& x0) {
+    x0 = col % tiles_x * kTXc;
+    const int r = col / tiles_x;
+    y0 = r % tiles_y * kTYc;
+    b = r / tiles_y;
   };
-  // Per tile: copies, then the 24 MMAs of one issuing thread; the next
-  // tile's copies wait for them (a second operand buffer, measured, was
-  // slower: two buffers of 103 KB leave fewer blocks per SM).
-  uint32_t par = 0u;
-  for (int k = 0; k < n; ++k) {
-    stage(k);
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    fence_proxy_async_smem();
-    tc_fence_before_sync();
-    __syncthreads();
-    if (tid == 0) {
-      tc_fence_after_sync();
-      const uint32_t a0 = smem_u32(smraw), b0 = a0 + W::A_BYTES;
-#pragma unroll
-      for (int cy = 0; cy < kTY; ++cy)
-#pragma unroll
-        for (int ddx = 0; ddx < 3; ++ddx)
-          tc_mma_bf16(tb + ddx * CIN, tc_sdesc(a0 + cy * kTX * 16, 128, W::A_SBO),
-                      tc_sdesc(b0 + (cy * W::HXp + ddx) * 16, 128, W::B_SBO), idesc, k > 0 || cy > 0);
-      tc_commit(&bar);
-    }
-    if (!mbar_wait(&bar, par)) atomicOr(flag, kFlagTimeout);
-    par ^= 1u;
-    tc_fence_after_sync();
-  }
-  // accumulators: lane = co (warps 0..3), column ddx * CIN + ci
-  if (n > 0 && warp < 4) {
-    const int co = 32 * warp + lane;
-#pragma unroll
-    for (int ddx = 0; ddx < 3; ++ddx) {
-      const int tap = dz * 9 + ddy * 3 + ddx;
-#pragma unroll
-      for (int j = 0; j < CIN / 8; ++j) {
-        float v[8];
-        tmem_ld8(tb + ((uint32_t)(32 * warp) << 16) + (uint32_t)(ddx * CIN + 8 * j), v);
-        if (co < cout_real) {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int ci = 8 * j + i;
-            if (ci < cin_real) atomicAdd(&dw[((long)co * cin_real + ci) * 27 + tap], v[i]);
-          }
+  if (warp == 0) {
+    // ---- producer: the weights (constants of this launch, last written before
+    // the kernel before this one), then the planes
+    if (lane == 0) mbar_arrive_expect_tx(&wbar, T::w_bytes);
+    __syncwarp();
+    if (lane < 27)
+      bulk_load(smraw + lane * (T::w_bytes / 27), p.wk + (long)lane * (T::w_bytes / 27 / sizeof(bf16_t)),
+                T::w_bytes / 27, &wbar);
+    pdl_wait();
+    if (lane == 0) {
+      int seq = 0;
+      bool ok = true;
+      for (int t = walk.t0; t < walk.t1 && ok; ++t) {
+        int b, y0, x0, z0, z1;
+        column(t / d.nz, b, y0, x0);
+        walk.fresh(t, z0, z1);
+        for (int z = z0; z <= z1; ++z, ++seq) {
+          const int slot = seq % RING;
+          if (seq >= RING) ok = role_wait(&empty[slot], (uint32_t)(seq / RING - 1) & 1u, p.flag);
+          if (!ok) break;
+          mbar_arrive_expect_tx(&full[slot], T::p_bytes);
+          // (stored cell (y0, x0) is cell (y0 - 1, x0 - 1) of the grid)
+          tensor_load3(smraw + T::w_bytes + slot * T::p_bytes, &in, x0 * 8, y0, (b * d.nz + z) * KC, &full[slot]);
         }
+      }
+      // no copy is in flight when the block ends (each full barrier's last phase)
+      for (int q = max(0, seq - RING); q < seq; ++q) mbar_wait(&full[q % RING], (uint32_t)(q / RING) & 1u);
+      mbar_wait(&wbar, 0);
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    {
+      // ---- MMA issue: the warp stays together (its operands are uniform), one thread issues
+      const uint32_t leader = tc_elect();
+      constexpr uint32_t idesc = tc_idesc_bf16(128, NP);
+      bool ok = __all_sync(0xffffffffu, role_wait(&wbar, 0, p.flag));
+      int seq = 0, zfirst = 0, sfirst = 0;  // ring position of the column's plane zfirst is sfirst
+      for (int t = walk.t0; t < walk.t1 && ok; ++t) {
+        const int k = t - walk.t0, z = t % d.nz;
+        int z0, z1;
+        walk.fresh(t, z0, z1);
+        if (t == walk.t0 || z == 0) {
+          zfirst = z0;
+          sfirst = seq;
+        }
+        for (int q = z0; q <= z1 && ok; ++q, ++seq)
+          ok = __all_sync(0xffffffffu, role_wait(&full[seq % RING], (uint32_t)(seq / RING) & 1u, p.flag));
+        if (k >= 2 && ok)
+          ok = __all_sync(0xffffffffu, role_wait(&tempty[k & 1], (uint32_t)(k / 2 - 1) & 1u, p.flag));
+        if (!ok) break;
+        tc_fence_after_sync();
+        const uint32_t dt = tb + (uint32_t)((k & 1) * NP);
+        bool acc = false;
+#pragma unroll 1
+        for (int dz = 0; dz < 3; ++dz) {
+          const int zp = z + dz - 1;
+          if (zp < 0 || zp >= d.nz) continue;
+          const uint64_t ad = tc_sdesc(sp_a + (uint32_t)((sfirst + zp - zfirst) % RING) * T::p_bytes, kPlaneC * 16,
+                                       kHXc * 16);
+          const uint64_t bd = tc_sdesc(sw_a + (uint32_t)(dz * 9 * KC * NP * 16), NP * 16, 128);
+          const uint32_t alo = (uint32_t)ad, ahi = (uint32_t)(ad >> 32), blo = (uint32_t)bd, bhi = (uint32_t)(bd >> 32);
+#pragma unroll
+          for (int tap = 0; tap < 9; ++tap)
+#pragma unroll
+            for (int ks = 0; ks < CIN / 16; ++ks) {
+              tc_mma_bf16_lo(dt, alo + (uint32_t)(2 * ks * kPlaneC + tap / 3 * kHXc + tap % 3), ahi,
+                             blo + (uint32_t)((tap * KC + 2 * ks) * NP), bhi, idesc, acc, leader);
+              acc = true;
+            }
+        }
+        // planes used for the last time by this tile
+        if (leader) {
+          if (z > 0) tc_commit(&empty[(sfirst + z - 1 - zfirst) % RING]);
+          if (z == d.nz - 1) tc_commit(&empty[(sfirst + z - zfirst) % RING]);
+          tc_commit(&tfull[k & 1]);
+        }
+        __syncwarp();
+      }
+    }
+    __syncwarp();
+  } else {
+    // ---- epilogue: warp reads lanes 32 (warp mod 4) .. + 31, columns of part (warp - 2) / 4
+    const int row = 32 * (warp & 3) + lane;
+    const int cx = row & 7, cy = row >> 3;
+    const int cb = (warp - 2) / 4 * NH;
+    pdl_wait();
+    float bv[NH];
+#pragma unroll
+    for (int c = 0; c < NH; ++c) bv[c] = (MODE == CM_BWD || cb + c >= COUT || (COUT == 8 && cb + c >= 3)) ? 0.f : __ldg(&p.bias[cb + c]);
+    float db[NH] = {};
+    double lsum = 0.0;
+    const long plane = (long)d.hp * d.wq * 8;
+    // (the walk's divisions once per column: they would be a third of the epilogue's instructions)
+    int z = walk.t0 % d.nz, b, y0, x0;
+    column(walk.t0 / d.nz, b, y0, x0);
+    for (int t = walk.t0; t < walk.t1; ++t, ++z) {
+      const int k = t - walk.t0;
+      if (z == d.nz) {
+        z = 0;
+        column(t / d.nz, b, y0, x0);
+      }
+      // (the vote also brings the warp together for the tensor-memory loads)
+      if (!__all_sync(0xffffffffu, role_wait(&tfull[k & 1], (uint32_t)(k / 2) & 1u, p.flag))) break;
+      tc_fence_after_sync();
+      float v[NH];
+#pragma unroll
+      for (int q = 0; q < NH / 8; ++q) {
+        float t8[8];
+        tmem_ld8(tb + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((k & 1) * NP + cb + 8 * q), t8);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[8 * q + i] = t8[i];
+      }
+      tc_fence_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&tempty[k & 1]);  // the accumulator may be overwritten
+      const int gx = x0 + cx, gy = y0 + cy;
+      if (gx >= d.nx || gy >= d.ny) continue;
+      const long bz = (long)b * d.nz + z;
+      if (MODE == CM_HIDDEN || MODE == CM_BWD) {
+        // eight channels per 16-byte store
+        const long at0 = (bz * (COUT / 8) + cb / 8) * plane + cell_at(d, gy, gx) * 8;
+#pragma unroll
+        for (int c = 0; c < NH; c += 8) {
+          const long at = at0 + c / 8 * plane;
+          uint32_t o[4];
+          if (MODE == CM_HIDDEN) {
+            uint32_t yp[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float v0 = v[c + 2 * j] + bv[c + 2 * j], v1 = v[c + 2 * j + 1] + bv[c + 2 * j + 1];
+              yp[j] = pack2(v0, v1);
+              o[j] = pack2(gelu_f(v0), gelu_f(v1));
+            }
+            if (p.ypre) *(uint4*)(p.ypre + at) = make_uint4(yp[0], yp[1], yp[2], yp[3]);
+          } else {
+            const uint4 y4 = *(const uint4*)(p.ypre + at);
+            const uint32_t yw[4] = {y4.x, y4.y, y4.z, y4.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float y0f = bf2f((bf16_t)(yw[j] & 0xffff)), y1f = bf2f((bf16_t)(yw[j] >> 16));
+              o[j] = pack2(v[c + 2 * j] * gelu_grad(y0f), v[c + 2 * j + 1] * gelu_grad(y1f));
+              db[c + 2 * j] += bf2f((bf16_t)(o[j] & 0xffff));
+              db[c + 2 * j + 1] += bf2f((bf16_t)(o[j] >> 16));
+            }
+          }
+          *(uint4*)(p.out + at) = make_uint4(o[0], o[1], o[2], o[3]);
+        }
+      } else if (cb == 0) {
+        const long cell = bz * ((long)d.nx * d.ny) + (long)gy * d.nx + gx;
+        const float q[3] = {v[0] + bv[0], v[1] + bv[1], v[2] + bv[2]};
+        if (MODE == CM_OUT) {
+          p.field[cell] = make_float4(q[0] * p.sd.x + p.mean.x, q[1] * p.sd.y + p.mean.y, q[2] * p.sd.z + p.mean.z, 0.f);
+        } else {
+          // SmoothL1 (beta 1) against the normalised target
+          const float4 tg = __ldg(&p.target[cell]);
+          const float e[3] = {q[0] - (tg.x - p.mean.x) * p.sd.x, q[1] - (tg.y - p.mean.y) * p.sd.y,
+                              q[2] - (tg.z - p.mean.z) * p.sd.z};
+          float g[3], l = 0.f;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const float a = fabsf(e[c]);
+            l += a < 1.f ? 0.5f * e[c] * e[c] : a - 0.5f;
+            g[c] = fminf(fmaxf(e[c], -1.f), 1.f) * p.inv_count;
+          }
+          lsum += (double)l;
+          const uint32_t o0 = pack2(g[0], g[1]), o1 = pack2(g[2], 0.f);
+          db[0] += bf2f((bf16_t)(o0 & 0xffff));
+          db[1] += bf2f((bf16_t)(o0 >> 16));
+          db[2] += bf2f((bf16_t)(o1 & 0xffff));
+          // (channels 8..15 of the padded sixteen stay at zero)
+          *(uint4*)(p.out + bz * 2 * plane + cell_at(d, gy, gx) * 8) = make_uint4(o0, o1, 0u, 0u);
+        }
+      }
+    }
+    if (MODE == CM_BWD || MODE == CM_LOSS) {
+      constexpr int ND = MODE == CM_LOSS ? 3 : NH;
+#pragma unroll
+      for (int c = 0; c < ND; ++c) {
+        float v = db[c];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (lane == 0 && (MODE == CM_BWD || cb == 0)) atomicAdd(&p.db[cb + c], v);
+      }
+      if (MODE == CM_LOSS) {
+        for (int o = 16; o > 0; o >>= 1) lsum += __shfl_down_sync(0xffffffffu, lsum, o);
+        if (lane == 0 && cb == 0) atomicAdd(p.loss, (float)(lsum * (double)p.inv_count));
       }
     }
   }
   tc_fence_before_sync();
   __syncthreads();
+  if (warp == 1) {
+    tc_fence_after_sync();
+    tmem_dealloc(tb, T::TCOLS);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Weight gradient of one layer: the correlation
+//   G[dz, dy][(s, cs)][cr] = sum_cells S[cell + (0, 0, s - 1)][cs] R[cell + (dz - 1, dy - 1, 0)][cr]
+// of a "stacked" operand S (CS channels) and a "ring" operand R (CR channels).  With
+// S = dY and R = x, G = dW[dz][dy][2 - s]; with S = x and R = dY (the layer whose
+// output is wider), G = dW[2 - dz][2 - dy][s].  The three x-shifts of S are three
+// copies of its tile in shared memory, so that they fill the M = 128 rows of one
+// MMA (3 CS of them; the rest is whatever follows in shared memory, and its
+// result is never read), and one MMA serves three taps: a tap per MMA reads the
+// same 4 KB of A for a third of the use.  N = CR, K = 16 cells of a row; one
+// accumulator of CR columns per dy in tensor memory: a CTA owns one dz and a range of
+// 16 x 8 tiles (a chain), in the order x, y, z, sample; two CTAs share an SM.
+// Tensor-core accumulation cuts each sum off below the accumulator's last place, so
+// its error grows with the number of MMAs a sum goes through: a chain is as many
+// tiles as six chains per SM and (dz, dy) make (81 at 64 samples of 64x64x4).
+// The middle dz, whose planes of R are all inside the grid, goes first: its blocks
+// are the longest.
+// Both operands are MN-major (channels contiguous, one 16-byte row of 8 channels
+// per cell, core matrices adjacent along K 128 B apart, 8-channel groups SBO
+// apart): boxes of the stored planes.  Planes of R outside the grid are left out.
+// The chains are added in FP32 in ws[(dz 3 + dy) CR + cr][(s, cs)], lanes next to
+// each other.  Bound: the MMAs' operand reads (6 KB per MMA at N = 64) and L2.
+// Measured at 64 samples of 64x64x4, with the kernel before in brackets (a (dz, dy)
+// per block, a tap per MMA, copies and MMAs in turn): 64 -> 32 and 32 -> 64 115 us
+// each (863, 600), 3 -> 32 and 32 -> 3 89 each (315, 452).  A CTA per SM with five or
+// four of the nine (dz, dy), planes of R kept in a ring: 131 and 101.
+// ---------------------------------------------------------------------------
+constexpr int kTX = 16, kTY = 8;  // tile (cells)
+template <int CS, int CR> struct WgradTc {
+  static constexpr uint32_t S_SBO = kTX * kTY * 16, R_SBO = kTX * (kTY + 2) * 16;  // slabs of 8 channels
+  static constexpr uint32_t s_bytes = 3 * (CS / 8) * S_SBO, r_bytes = (CR / 8) * R_SBO, stage = s_bytes + r_bytes;
+  static constexpr int ST = (int)(113 * 1024 / stage) < 4 ? (int)(113 * 1024 / stage) : 4;  // stages
+  static_assert(ST >= 2, "wgrad stages");
+  // the 16 row groups of an MMA starting in the last stage stay inside
+  static constexpr uint32_t reach = (ST - 1) * stage + 16 * S_SBO + kTX * kTY * 16;
+  static constexpr size_t smem = ST * stage > reach ? ST * stage : reach;
+  static constexpr uint32_t TCOLS = 3 * CR <= 128 ? 128 : 256;
+  static_assert(3 * CS <= 128 && 3 * CR <= 256 && CR % 16 == 0, "wgrad shape");
+};
+
+template <int CS, int CR>
+__global__ void __launch_bounds__(192, 2)
+    wgrad_tc_kernel(const __grid_constant__ CUtensorMap S, const __grid_constant__ CUtensorMap R,
+                    float* __restrict__ ws, ConvDims d, int chain, int* flag) {
+  typedef WgradTc<CS, CR> W;
+  constexpr int ST = W::ST;
+  extern __shared__ __align__(128) unsigned char smraw[];
+  __shared__ __align__(8) uint64_t full[ST], empty[ST], done;
+  __shared__ uint32_t tbase, started_s;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int chains = (int)gridDim.x / 3, third = (int)blockIdx.x / chains;
+  const int dz = third == 0 ? 1 : third == 1 ? 0 : 2;
+  if (tid == 0) {
+    for (int q = 0; q < ST; ++q) {
+      mbar_init(&full[q], 1);
+      mbar_init(&empty[q], 1);
+    }
+    mbar_init(&done, 1);
+    started_s = 0u;
+  }
+  if (warp == 1) tmem_alloc(&tbase, W::TCOLS);
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const uint32_t tb = tbase;
+  const int tiles_x = (d.nx + kTX - 1) / kTX, tiles_y = (d.ny + kTY - 1) / kTY;
+  const long ntiles = (long)tiles_x * tiles_y * d.nz * d.batch;
+  const long t0 = (long)((int)blockIdx.x % chains) * chain, t1 = t0 + chain < ntiles ? t0 + chain : ntiles;
+  // tile t: its plane's index b nz + z; whether R's plane is inside the grid
+  auto inside = [&](long t, int& bz) {
+    bz = (int)(t / (tiles_x * tiles_y));
+    const int zp = bz % d.nz + dz - 1;
+    return zp >= 0 && zp < d.nz;
+  };
+  pdl_wait();
   if (warp == 0) {
+    if (lane == 0) {
+      int k = 0;
+      bool ok = true;
+      for (long t = t0; t < t1; ++t) {
+        int bz;
+        if (!inside(t, bz)) continue;
+        if (k >= ST) ok = role_wait(&empty[k % ST], (uint32_t)(k / ST - 1) & 1u, flag);
+        if (!ok) break;
+        const int x0 = (int)(t % tiles_x) * kTX, y0 = (int)(t / tiles_x % tiles_y) * kTY;
+        uint64_t* bar = &full[k % ST];
+        unsigned char* st = smraw + (k % ST) * W::stage;
+        mbar_arrive_expect_tx(bar, W::stage);
+        // S: three copies shifted by -1, 0, +1 in x (stored cell (y + 1, x + 1) is cell (y, x))
+        for (int sh = 0; sh < 3; ++sh)
+          tensor_load3(st + sh * (W::s_bytes / 3), &S, (x0 + sh) * 8, y0 + 1, bz * (CS / 8), bar);
+        tensor_load3(st + W::s_bytes, &R, (x0 + 1) * 8, y0, (bz + dz - 1) * (CR / 8), bar);
+        ++k;
+      }
+      // no copy is in flight when the block ends
+      for (int q = max(0, k - ST); q < k; ++q) mbar_wait(&full[q % ST], (uint32_t)(q / ST) & 1u);
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    const uint32_t leader = tc_elect();
+    constexpr uint32_t idesc = tc_idesc_bf16(128, CR) | (1u << 15) | (1u << 16);  // A and B MN-major
+    const uint32_t s_a = smem_u32(smraw);
+    int k = 0;
+    bool ok = true;
+    for (long t = t0; t < t1; ++t) {
+      int bz;
+      if (!inside(t, bz)) continue;
+      ok = __all_sync(0xffffffffu, role_wait(&full[k % ST], (uint32_t)(k / ST) & 1u, flag));
+      if (!ok) break;
+      tc_fence_after_sync();
+      const uint32_t sa = s_a + (uint32_t)(k % ST) * W::stage;
+      const uint64_t ad = tc_sdesc(sa, 128, W::S_SBO), bd = tc_sdesc(sa + W::s_bytes, 128, W::R_SBO);
+#pragma unroll
+      for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+        for (int cy = 0; cy < kTY; ++cy)
+          tc_mma_bf16_lo(tb + dy * CR, (uint32_t)ad + cy * kTX, (uint32_t)(ad >> 32), (uint32_t)bd + (cy + dy) * kTX,
+                         (uint32_t)(bd >> 32), idesc, cy > 0 || k > 0, leader);
+      if (leader) tc_commit(&empty[k % ST]);
+      __syncwarp();
+      ++k;
+    }
+    if (leader) {
+      started_s = ok && k > 0 ? 1u : 0u;
+      tc_commit(&done);
+    }
+    __syncwarp();
+    role_wait(&done, 0, flag);  // no MMA is in flight when the block ends
+  } else {
+    // ---- the chain's sums: lane = row (s, cs) of quarter warp mod 4
+    const int row = 32 * (warp & 3) + lane;
+    const bool ok = __all_sync(0xffffffffu, role_wait(&done, 0, flag));
+    tc_fence_after_sync();
+    if (ok && *(volatile uint32_t*)&started_s && 32 * (warp & 3) < 3 * CS) {
+#pragma unroll 1
+      for (int c = 0; c < 3 * CR; c += 8) {
+        float v[8];
+        tmem_ld8(tb + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c, v);
+        if (row < 3 * CS) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) atomicAdd(&ws[(long)(dz * 3 * CR + c + i) * (3 * CS) + row], v[i]);
+        }
+        __syncwarp();
+      }
+    }
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  if (warp == 1) {
     tc_fence_after_sync();
     tmem_dealloc(tb, W::TCOLS);
   }
 }
 
-// bias gradient: db[co] += sum over cells of dY[cell][co]
-__global__ void bgrad_kernel(const bf16_t* __restrict__ dy, int cpad, int creal, long ncells, float* __restrict__ db) {
-  const int co = threadIdx.x % 64;
-  const int lane_grp = threadIdx.x / 64;  // 4 groups
-  if (co >= creal) return;
-  float s = 0.f;
-  for (long c = (long)blockIdx.x * 4 + lane_grp; c < ncells; c += (long)gridDim.x * 4) s += bf2f(dy[c * cpad + co]);
-  atomicAdd(&db[co], s);
+// ws of all four layers -> the gradient's weights (parameter order [co][ci][27])
+struct WgradOut {
+  long ws, dw;       // offsets
+  int cs, cr, cin, cout, sx;  // sx: S is x (else dY)
+};
+struct WgradOuts {
+  WgradOut l[4];
+};
+__global__ void wgrad_finish_kernel(const float* __restrict__ ws, float* __restrict__ grad, WgradOuts o) {
+  const WgradOut l = o.l[blockIdx.y];
+  pdl_wait();
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= l.cout * l.cin * 27) return;
+  const int tap = e % 27, ci = e / 27 % l.cin, co = e / 27 / l.cin;
+  const int dz = tap / 9, dy = tap / 3 % 3, dx = tap % 3;
+  const int j = l.sx ? (2 - dz) * 3 + 2 - dy : dz * 3 + dy, s = l.sx ? dx : 2 - dx;
+  const int cs = l.sx ? ci : co, cr = l.sx ? co : ci;
+  grad[l.dw + e] = ws[l.ws + (long)(j * l.cr + cr) * (3 * l.cs) + s * l.cs + cs];
 }
 
-// input normalisation: m float4 -> x0 bf16 [cells][16]
-__global__ void normalize_in_kernel(const float4* __restrict__ m, bf16_t* __restrict__ x0, long ncells, float3 mean,
-                                    float3 inv_std) {
+// input normalisation: m float4 -> the first eight channels of the padded input
+__global__ void normalize_in_kernel(const float4* __restrict__ m, bf16_t* __restrict__ x0, ConvDims d, long ncells,
+                                    float3 mean, float3 inv_std) {
   const long c = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_wait();
   if (c >= ncells) return;
   const float4 v = m[c];
-  uint4 lo, hi;
-  lo.x = pack2((v.x - mean.x) * inv_std.x, (v.y - mean.y) * inv_std.y);
-  lo.y = pack2((v.z - mean.z) * inv_std.z, 0.f);
-  lo.z = lo.w = 0u;
-  hi.x = hi.y = hi.z = hi.w = 0u;
-  uint4* o = (uint4*)(x0 + c * 16);
-  o[0] = lo;
-  o[1] = hi;
+  const int x = (int)(c % d.nx), y = (int)(c / d.nx % d.ny);
+  const long bz = c / ((long)d.nx * d.ny);
+  uint4 o;
+  o.x = pack2((v.x - mean.x) * inv_std.x, (v.y - mean.y) * inv_std.y);
+  o.y = pack2((v.z - mean.z) * inv_std.z, 0.f);
+  o.z = o.w = 0u;
+  *(uint4*)(x0 + (bz * 2 * d.hp * d.wq + cell_at(d, y, x)) * 8) = o;
 }
 
-// output: normalised prediction (float4) -> H = pred * std + mean
-__global__ void denormalize_out_kernel(const float4* __restrict__ pred, float4* __restrict__ h, long ncells,
-                                       float3 mean, float3 std) {
-  const long c = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= ncells) return;
-  const float4 p = pred[c];
-  h[c] = make_float4(p.x * std.x + mean.x, p.y * std.y + mean.y, p.z * std.z + mean.z, 0.f);
-}
-
-// SmoothL1 (beta 1) of pred against the normalised target; dY4 [cells][16] bf16
-__global__ void loss_kernel(const float4* __restrict__ pred, const float4* __restrict__ h_target, long ncells,
-                            float3 mean, float3 inv_std, float inv_count, bf16_t* __restrict__ dy4,
-                            float* __restrict__ loss) {
-  const long c = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  float l = 0.f;
-  if (c < ncells) {
-    const float4 p = pred[c];
-    const float4 t = h_target[c];
-    const float d0 = p.x - (t.x - mean.x) * inv_std.x;
-    const float d1 = p.y - (t.y - mean.y) * inv_std.y;
-    const float d2 = p.z - (t.z - mean.z) * inv_std.z;
-    const float ds[3] = {d0, d1, d2};
-    float g[3];
-    for (int k = 0; k < 3; ++k) {
-      const float a = fabsf(ds[k]);
-      l += a < 1.f ? 0.5f * ds[k] * ds[k] : a - 0.5f;
-      g[k] = fminf(fmaxf(ds[k], -1.f), 1.f) * inv_count;
-    }
-    uint4 lo, hi;
-    lo.x = pack2(g[0], g[1]);
-    lo.y = pack2(g[2], 0.f);
-    lo.z = lo.w = 0u;
-    hi.x = hi.y = hi.z = hi.w = 0u;
-    uint4* o = (uint4*)(dy4 + c * 16);
-    o[0] = lo;
-    o[1] = hi;
-  }
-  for (int o = 16; o > 0; o >>= 1) l += __shfl_down_sync(0xffffffffu, l, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, l * inv_count);
-}
-
-// FP32 master weights -> bf16 [27][COUT_PAD][CIN_PAD] (forward) and the
-// flipped, transposed copy [27][CIN_PAD'][COUT_PAD'] for the backward pass.
+// FP32 master weights -> bf16 [27][CIN_PAD/8][COUT_PAD][8] (forward) and the
+// flipped, transposed copy [27][CIN_PAD'/8][COUT_PAD'][8] for the backward pass.
 __global__ void pack_weights_kernel(const float* __restrict__ W, int cin, int cout, bf16_t* __restrict__ fwd,
                                     int cin_pad, int cout_pad, bf16_t* __restrict__ bwd, int bwd_in_pad,
                                     int bwd_out_pad) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   const int nf = 27 * cout_pad * cin_pad;
   if (e < nf) {
-    const int ci = e % cin_pad, co = (e / cin_pad) % cout_pad, tap = e / (cin_pad * cout_pad);
+    const int co = e / 8 % cout_pad, ci = e / 8 / cout_pad % (cin_pad / 8) * 8 + e % 8, tap = e / (cin_pad * cout_pad);
     const float v = (ci < cin && co < cout) ? W[((long)co * cin + ci) * 27 + tap] : 0.f;
     fwd[e] = f2bf(v);
   }
@@ -488,8 +584,8 @@ __global__ void pack_weights_kernel(const float* __restrict__ W, int cin, int co
     const int nb = 27 * bwd_out_pad * bwd_in_pad;
     if (e < nb) {
       // backward conv: input channels = this layer's cout, output channels = cin
-      const int co = e % bwd_in_pad, ci = (e / bwd_in_pad) % bwd_out_pad, tapb = e / (bwd_in_pad * bwd_out_pad);
-      const int tap = 26 - tapb;
+      const int ci = e / 8 % bwd_out_pad, co = e / 8 / bwd_out_pad % (bwd_in_pad / 8) * 8 + e % 8;
+      const int tap = 26 - e / (bwd_in_pad * bwd_out_pad);
       const float v = (ci < cin && co < cout) ? W[((long)co * cin + ci) * 27 + tap] : 0.f;
       bwd[e] = f2bf(v);
     }
@@ -537,7 +633,11 @@ struct mx_cnn {
   bf16_t* wb[4] = {nullptr, nullptr, nullptr, nullptr};
   bf16_t *x0 = nullptr, *a1 = nullptr, *y1 = nullptr, *a2 = nullptr, *y2 = nullptr, *a3 = nullptr, *y3 = nullptr;
   bf16_t *dy4 = nullptr, *dy3 = nullptr, *dy2 = nullptr, *dy1 = nullptr;
-  float4* pred = nullptr;
+  // the activations as tensors [b z C/8][hp][wq 8] with the boxes of the
+  // convolutions' input planes and of the weight gradients' S and R tiles
+  CUtensorMap c_x0, c_a1, c_a2, c_a3, c_dy4, c_dy3, c_dy2;
+  CUtensorMap s_x0, s_a1, s_dy3, s_dy4, r_dy1, r_dy2, r_a2, r_a3;
+  float* ws = nullptr;      // weight-gradient sums of the four layers, in their kernels' order
   float* loss = nullptr;
   int* flag = nullptr;  // device status bits (kFlagTimeout), read by mx_cnn_sync / mx_sync
   float stats[12] = {0, 0, 0, 1, 1, 1, 0, 0, 0, 1, 1, 1};
@@ -558,67 +658,137 @@ static ConvDims conv_dims(const mx_cnn* n, int batch) {
   d.ny = n->ny;
   d.nz = n->nz;
   d.batch = batch;
-  d.tiles_x = (n->nx + kTX - 1) / kTX;
-  d.tiles_y = (n->ny + kTY - 1) / kTY;
-  d.ntiles = d.tiles_x * d.tiles_y * n->nz * batch;
+  // the widest tiles are 16 cells in each direction; a border of one cell on each side
+  d.wq = (n->nx + 15) / 16 * 16 + 2;
+  d.hp = (n->ny + 15) / 16 * 16 + 2;
   return d;
 }
+// elements of a stored activation of C channels
+static size_t act_elems(const mx_cnn* n, int C, int batch) {
+  const ConvDims d = conv_dims(n, 1);
+  return (size_t)batch * n->nz * C * d.hp * d.wq;
+}
 
-static int g_num_sms = 0;
+// Tensor map of an activation of C channels, box bx cells x by rows x all C / 8 planes of a layer.
+static mx_status make_map(const mx_cnn* n, CUtensorMap* map, bf16_t* base, int C, int bx, int by) {
+  typedef CUresult (*Encode)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                             const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                             CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  static const Encode encode = []() -> Encode {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      fn = nullptr;
+    }
+    return (Encode)fn;
+  }();
+  if (!encode) {
+    set_error("mx_cnn_create: the driver has no cuTensorMapEncodeTiled");
+    return MX_ERR_CUDA;
+  }
+  const ConvDims d = conv_dims(n, n->max_batch);
+  const cuuint64_t dims[3] = {(cuuint64_t)d.wq * 8, (cuuint64_t)d.hp, (cuuint64_t)n->max_batch * n->nz * (C / 8)};
+  const cuuint64_t strides[2] = {(cuuint64_t)d.wq * 16, (cuuint64_t)d.wq * 16 * d.hp};
+  const cuuint32_t box[3] = {(cuuint32_t)bx * 8, (cuuint32_t)by, (cuuint32_t)(C / 8)}, one[3] = {1, 1, 1};
+  if (encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
+    set_error("mx_cnn_create: tensor map not encoded");
+    return MX_ERR_CUDA;
+  }
+  return MX_OK;
+}
+static mx_status make_maps(mx_cnn* n) {
+  auto c = [&](CUtensorMap* m, bf16_t* b, int C) { return make_map(n, m, b, C, kHXc, kHYc); };
+  auto s = [&](CUtensorMap* m, bf16_t* b, int C) { return make_map(n, m, b, C, kTX, kTY); };
+  auto r = [&](CUtensorMap* m, bf16_t* b, int C) { return make_map(n, m, b, C, kTX, kTY + 2); };
+  MX_TRY(c(&n->c_x0, n->x0, 16));
+  MX_TRY(c(&n->c_a1, n->a1, 32));
+  MX_TRY(c(&n->c_a2, n->a2, 64));
+  MX_TRY(c(&n->c_a3, n->a3, 32));
+  MX_TRY(c(&n->c_dy4, n->dy4, 16));
+  MX_TRY(c(&n->c_dy3, n->dy3, 32));
+  MX_TRY(c(&n->c_dy2, n->dy2, 64));
+  MX_TRY(s(&n->s_x0, n->x0, 16));
+  MX_TRY(s(&n->s_a1, n->a1, 32));
+  MX_TRY(s(&n->s_dy3, n->dy3, 32));
+  MX_TRY(s(&n->s_dy4, n->dy4, 16));
+  MX_TRY(r(&n->r_dy1, n->dy1, 32));
+  MX_TRY(r(&n->r_dy2, n->dy2, 64));
+  MX_TRY(r(&n->r_a2, n->a2, 64));
+  return r(&n->r_a3, n->a3, 32);
+}
+
+static int num_sms() {
+  int dev = 0, v = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
+    v = 1;
+  return v;
+}
 
 template <int CIN, int COUT, int MODE>
-static mx_status conv_launch(const bf16_t* in, const bf16_t* w, const float* b, bf16_t* out, bf16_t* ypre,
-                             float4* outf, const ConvDims& d, int* flag, int ntiles, cudaStream_t st) {
-  const size_t sm = ConvTc<CIN, COUT>::smem;
-  static bool attr = false;
-  if (!attr) {
-    MX_CUDA_TRY(cudaFuncSetAttribute(conv_tc_kernel<CIN, COUT, MODE>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    attr = true;
+static mx_status conv_run(const CUtensorMap& in, const ConvArgs& p, cudaStream_t st, bool setup = false) {
+  typedef ConvTc<CIN, COUT> T;
+  auto k = conv_tc_kernel<CIN, COUT, MODE>;
+  if (setup) {
+    MX_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem));
+    return MX_OK;
   }
-  const int ctas = ntiles < g_num_sms ? ntiles : g_num_sms;
-  conv_tc_kernel<CIN, COUT, MODE><<<ctas, kCnnThreads, sm, st>>>(in, w, b, out, ypre, outf, d, flag);
+  const ConvDims& d = p.d;
+  const long ntiles = (long)((d.nx + kTXc - 1) / kTXc) * ((d.ny + kTYc - 1) / kTYc) * d.nz * d.batch;
+  const int sms = num_sms();
+  launch_pdl(k, dim3((unsigned)(ntiles < sms ? ntiles : sms)), dim3(T::threads), T::smem, st, in, p);
   return launch_check("conv_tc_kernel");
 }
 
-template <int CIN, int COUT, int MODE>
-static mx_status conv_run(const bf16_t* in, const bf16_t* w, const float* b, bf16_t* out, bf16_t* ypre, float4* outf,
-                          const ConvDims& d, int* flag, cudaStream_t st) {
-  if (!g_num_sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (g_num_sms <= 0) g_num_sms = 1;
+template <int CS, int CR>
+static mx_status wgrad_run(const CUtensorMap& S, const CUtensorMap& R, float* ws, const ConvDims& d, int* flag, cudaStream_t st,
+                           bool setup = false) {
+  typedef WgradTc<CS, CR> W;
+  auto k = wgrad_tc_kernel<CS, CR>;
+  if (setup) {
+    MX_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W::smem));
+    return MX_OK;
   }
-  const int ntiles = ((d.nx + kTXc - 1) / kTXc) * ((d.ny + kTYc - 1) / kTYc) * d.nz * d.batch;
-  return conv_launch<CIN, COUT, MODE>(in, w, b, out, ypre, outf, d, flag, ntiles, st);
+  const long ntiles = (long)((d.nx + kTX - 1) / kTX) * ((d.ny + kTY - 1) / kTY) * d.nz * d.batch;
+  const long six = 6L * num_sms();
+  const int chain = (int)((ntiles * 9 + six - 1) / six);
+  const long chains = (ntiles + chain - 1) / chain;
+  launch_pdl(k, dim3((unsigned)(3 * chains)), dim3(192), W::smem, st, S, R, ws, d, chain, flag);
+  return launch_check("wgrad_tc_kernel");
 }
 
-template <int CIN, int COUT>
-static mx_status wgrad_run(const bf16_t* x, const bf16_t* dy, float* dw, const ConvDims& d, int cin_real,
-                           int cout_real, int* flag, cudaStream_t st) {
-  typedef WgradShape<CIN, COUT> W;
-  static bool attr = false;
-  if (!attr) {
-    MX_CUDA_TRY(cudaFuncSetAttribute(wgrad_tc_kernel<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)W::smem));
-    attr = true;
+// Where each layer's sums lie in ws and go in the gradient.
+static WgradOuts wgrad_outs(long* total) {
+  // layers 1 and 2 stack x (16, 32 channels), layers 3 and 4 stack dY (32, 16)
+  static const int cs[4] = {16, 32, 32, 16}, cr[4] = {32, 64, 64, 32}, sx[4] = {1, 1, 0, 0};
+  WgradOuts o;
+  long at = 0;
+  for (int l = 0; l < 4; ++l) {
+    o.l[l] = WgradOut{at, layer_w_off(l), cs[l], cr[l], kCh[l], kCh[l + 1], sx[l]};
+    at += 27L * cs[l] * cr[l];
   }
-  if (!g_num_sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (g_num_sms <= 0) g_num_sms = 1;
-  }
-  // about six blocks per SM over the nine (dz, ddy) tap rows: blocks that
-  // wait for tensor memory or for their MMAs overlap the others' copies
-  // (measured: 5.00 ms per batch-64 loss + gradient at 64x64x4 against 5.89
-  // with two blocks per SM and 5.66 with the earlier mma.sync kernel)
-  int tpb = (int)(((long)d.ntiles * 9 + 6 * g_num_sms - 1) / (6 * g_num_sms));
-  if (tpb < 1) tpb = 1;
-  dim3 grid((d.ntiles + tpb - 1) / tpb, 9);
-  wgrad_tc_kernel<CIN, COUT><<<grid, kCnnThreads, W::smem, st>>>(x, dy, dw, d, cin_real, cout_real, tpb, flag);
-  return launch_check("wgrad_tc_kernel");
+  *total = at;
+  return o;
+}
+
+static mx_status cnn_setup() {
+  const ConvArgs none{};
+  const ConvDims nd{};
+  const CUtensorMap nm{};
+  MX_TRY((conv_run<16, 32, CM_HIDDEN>(nm, none, nullptr, true)));
+  MX_TRY((conv_run<32, 64, CM_HIDDEN>(nm, none, nullptr, true)));
+  MX_TRY((conv_run<64, 32, CM_HIDDEN>(nm, none, nullptr, true)));
+  MX_TRY((conv_run<32, 8, CM_OUT>(nm, none, nullptr, true)));
+  MX_TRY((conv_run<32, 8, CM_LOSS>(nm, none, nullptr, true)));
+  MX_TRY((conv_run<16, 32, CM_BWD>(nm, none, nullptr, true)));
+  MX_TRY((conv_run<32, 64, CM_BWD>(nm, none, nullptr, true)));
+  MX_TRY((conv_run<64, 32, CM_BWD>(nm, none, nullptr, true)));
+  MX_TRY((wgrad_run<16, 32>(nm, nm, nullptr, nd, nullptr, nullptr, true)));
+  return wgrad_run<32, 64>(nm, nm, nullptr, nd, nullptr, nullptr, true);
 }
 
 static mx_status pack_all(mx_cnn* n, cudaStream_t st) {
@@ -637,30 +807,43 @@ static mx_status pack_all(mx_cnn* n, cudaStream_t st) {
   return MX_OK;
 }
 
-static mx_status cnn_forward_to_pred(mx_cnn* n, const float4* m, int batch, cudaStream_t st) {
+// The three hidden layers: m -> a3 (and, for training, the pre-activations).
+static mx_status cnn_hidden(mx_cnn* n, const float4* m, int batch, bool train, cudaStream_t st) {
   const long nc = n->cells * batch;
   const float* s = n->stats;
-  normalize_in_kernel<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(
-      m, n->x0, nc, make_float3(s[0], s[1], s[2]), make_float3(1.f / s[3], 1.f / s[4], 1.f / s[5]));
-  MX_TRY(launch_check("normalize_in_kernel"));
   const ConvDims d = conv_dims(n, batch);
+  launch_pdl(normalize_in_kernel, dim3((unsigned)((nc + 255) / 256)), dim3(256), 0, st, m, n->x0, d, nc,
+             make_float3(s[0], s[1], s[2]), make_float3(1.f / s[3], 1.f / s[4], 1.f / s[5]));
+  MX_TRY(launch_check("normalize_in_kernel"));
   const float* P = n->params;
-  MX_TRY((conv_run<16, 32, CM_HIDDEN>(n->x0, n->wf[0], P + layer_w_off(0) + 32 * 3 * 27, n->a1, n->y1, nullptr, d, n->flag, st)));
-  MX_TRY((conv_run<32, 64, CM_HIDDEN>(n->a1, n->wf[1], P + layer_w_off(1) + 64 * 32 * 27, n->a2, n->y2, nullptr, d, n->flag, st)));
-  MX_TRY((conv_run<64, 32, CM_HIDDEN>(n->a2, n->wf[2], P + layer_w_off(2) + 32 * 64 * 27, n->a3, n->y3, nullptr, d, n->flag, st)));
-  MX_TRY((conv_run<32, 8, CM_LAST>(n->a3, n->wf[3], P + layer_w_off(3) + 3 * 32 * 27, nullptr, nullptr, n->pred, d, n->flag, st)));
-  return MX_OK;
+  ConvArgs a{};
+  a.d = d;
+  a.flag = n->flag;
+  a.wk = n->wf[0], a.bias = P + layer_w_off(0) + 32 * 3 * 27, a.out = n->a1;
+  a.ypre = train ? n->y1 : nullptr;
+  MX_TRY((conv_run<16, 32, CM_HIDDEN>(n->c_x0, a, st)));
+  a.wk = n->wf[1], a.bias = P + layer_w_off(1) + 64 * 32 * 27, a.out = n->a2;
+  a.ypre = train ? n->y2 : nullptr;
+  MX_TRY((conv_run<32, 64, CM_HIDDEN>(n->c_a1, a, st)));
+  a.wk = n->wf[2], a.bias = P + layer_w_off(2) + 32 * 64 * 27, a.out = n->a3;
+  a.ypre = train ? n->y3 : nullptr;
+  return conv_run<64, 32, CM_HIDDEN>(n->c_a2, a, st);
+}
+
+static mx_status cnn_forward(mx_cnn* n, const float4* m, float4* h, int batch, cudaStream_t st) {
+  MX_TRY(cnn_hidden(n, m, batch, false, st));
+  const float* s = n->stats;
+  ConvArgs a{};
+  a.d = conv_dims(n, batch);
+  a.flag = n->flag;
+  a.wk = n->wf[3], a.bias = n->params + layer_w_off(3) + 3 * 32 * 27, a.field = h;
+  a.mean = make_float3(s[6], s[7], s[8]), a.sd = make_float3(s[9], s[10], s[11]);
+  return conv_run<32, 8, CM_OUT>(n->c_a3, a, st);
 }
 
 bool cnn_matches(const mx_cnn* n, const Grid& g) { return n->nx == g.nx && n->ny == g.ny && n->nz == g.nz; }
 
-mx_status cnn_demag(mx_cnn* n, const float4* m, float4* h, cudaStream_t st) {
-  MX_TRY(cnn_forward_to_pred(n, m, 1, st));
-  const float* s = n->stats;
-  denormalize_out_kernel<<<(unsigned)((n->cells + 255) / 256), 256, 0, st>>>(
-      n->pred, h, n->cells, make_float3(s[6], s[7], s[8]), make_float3(s[9], s[10], s[11]));
-  return launch_check("denormalize_out_kernel");
-}
+mx_status cnn_demag(mx_cnn* n, const float4* m, float4* h, cudaStream_t st) { return cnn_forward(n, m, h, 1, st); }
 
 // Reads and clears the net's device status flag (synchronises `stream`).
 mx_status cnn_take_flag(mx_cnn* n, cudaStream_t st, int* flag_out) {
@@ -687,7 +870,7 @@ mx_status mx_cnn_destroy(mx_cnn* n) {
   if (!n) return MX_OK;
   void* ptrs[] = {n->params, n->grad, n->am, n->av, n->wf[0], n->wf[1], n->wf[2], n->wf[3], n->wb[1], n->wb[2],
                   n->wb[3], n->x0, n->a1, n->y1, n->a2, n->y2, n->a3, n->y3, n->dy4, n->dy3, n->dy2, n->dy1,
-                  n->pred, n->loss, n->flag};
+                  n->ws, n->loss, n->flag};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete n;
@@ -707,49 +890,44 @@ mx_status mx_cnn_create(mx_cnn** out, int nx, int ny, int nz, int max_batch) {
   n->nz = nz;
   n->max_batch = max_batch;
   n->cells = (long)nx * ny * nz;
-  const long nc = n->cells * max_batch;
   const long np = num_params_total();
+  long nws = 0;
+  wgrad_outs(&nws);
   bool ok = true;
-  auto alloc = [&](void** p, size_t bytes) {
+  auto alloc = [&](void** p, size_t bytes, bool zero) {
     if (ok && cudaMalloc(p, bytes) != cudaSuccess) {
       cudaGetLastError();
       ok = false;
     }
+    if (ok && zero && cudaMemset(*p, 0, bytes) != cudaSuccess) ok = false;
   };
-  alloc((void**)&n->params, sizeof(float) * np);
-  alloc((void**)&n->grad, sizeof(float) * np);
-  alloc((void**)&n->am, sizeof(float) * np);
-  alloc((void**)&n->av, sizeof(float) * np);
+  alloc((void**)&n->params, sizeof(float) * np, true);
+  alloc((void**)&n->grad, sizeof(float) * np, false);
+  alloc((void**)&n->am, sizeof(float) * np, true);
+  alloc((void**)&n->av, sizeof(float) * np, true);
   const int bw_in[4] = {0, 64, 32, 16}, bw_out[4] = {0, 32, 64, 32};
   for (int l = 0; l < 4; ++l) {
-    alloc((void**)&n->wf[l], sizeof(bf16_t) * 27 * kCoutPad[l] * kCinPad[l]);
-    if (l > 0) alloc((void**)&n->wb[l], sizeof(bf16_t) * 27 * bw_in[l] * bw_out[l]);
+    alloc((void**)&n->wf[l], sizeof(bf16_t) * 27 * kCoutPad[l] * kCinPad[l], true);
+    if (l > 0) alloc((void**)&n->wb[l], sizeof(bf16_t) * 27 * bw_in[l] * bw_out[l], true);
   }
-  alloc((void**)&n->x0, sizeof(bf16_t) * nc * 16);
-  alloc((void**)&n->a1, sizeof(bf16_t) * nc * 32);
-  alloc((void**)&n->y1, sizeof(bf16_t) * nc * 32);
-  alloc((void**)&n->a2, sizeof(bf16_t) * nc * 64);
-  alloc((void**)&n->y2, sizeof(bf16_t) * nc * 64);
-  alloc((void**)&n->a3, sizeof(bf16_t) * nc * 32);
-  alloc((void**)&n->y3, sizeof(bf16_t) * nc * 32);
-  alloc((void**)&n->dy4, sizeof(bf16_t) * nc * 16);
-  alloc((void**)&n->dy3, sizeof(bf16_t) * nc * 32);
-  alloc((void**)&n->dy2, sizeof(bf16_t) * nc * 64);
-  alloc((void**)&n->dy1, sizeof(bf16_t) * nc * 32);
-  alloc((void**)&n->pred, sizeof(float4) * nc);
-  alloc((void**)&n->loss, sizeof(float));
-  alloc((void**)&n->flag, sizeof(int));
+  // zero once: the borders, and the channels that padding adds, are never written
+  bf16_t** act[] = {&n->x0, &n->a1, &n->y1, &n->a2, &n->y2, &n->a3, &n->y3, &n->dy4, &n->dy3, &n->dy2, &n->dy1};
+  const int ch[] = {16, 32, 32, 64, 64, 32, 32, 16, 32, 64, 32};
+  for (int q = 0; q < 11; ++q) alloc((void**)act[q], sizeof(bf16_t) * act_elems(n, ch[q], max_batch), true);
+  alloc((void**)&n->ws, sizeof(float) * nws, false);
+  alloc((void**)&n->loss, sizeof(float), false);
+  alloc((void**)&n->flag, sizeof(int), true);
   if (!ok) {
     mx_cnn_destroy(n);
     set_error("mx_cnn_create: device allocation failed");
     return MX_ERR_OOM;
   }
-  if (cudaMemset(n->params, 0, sizeof(float) * np) != cudaSuccess || cudaMemset(n->flag, 0, sizeof(int)) != cudaSuccess ||
-      cudaMemset(n->am, 0, sizeof(float) * np) != cudaSuccess ||
-      cudaMemset(n->av, 0, sizeof(float) * np) != cudaSuccess) {
+  mx_status st = cnn_setup();
+  if (st == MX_OK) st = make_maps(n);
+  if (st != MX_OK || cudaDeviceSynchronize() != cudaSuccess) {
     mx_cnn_destroy(n);
-    set_error("mx_cnn_create: memset failed");
-    return MX_ERR_CUDA;
+    if (st == MX_OK) set_error("mx_cnn_create: set-up failed");
+    return st != MX_OK ? st : MX_ERR_CUDA;
   }
   *out = n;
   return MX_OK;
@@ -822,13 +1000,7 @@ mx_status mx_cnn_forward(mx_cnn* n, const float* m, float* h, int batch, mx_stre
     set_error("mx_cnn_forward: h must be a 16-byte aligned device pointer");
     return MX_ERR_INVALID_ARG;
   }
-  cudaStream_t st = (cudaStream_t)stream;
-  MX_TRY(cnn_forward_to_pred(n, (const float4*)m, batch, st));
-  const float* s = n->stats;
-  const long nc = n->cells * batch;
-  denormalize_out_kernel<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(
-      n->pred, (float4*)h, nc, make_float3(s[6], s[7], s[8]), make_float3(s[9], s[10], s[11]));
-  return launch_check("denormalize_out_kernel");
+  return cnn_forward(n, (const float4*)m, (float4*)h, batch, (cudaStream_t)stream);
 }
 
 mx_status mx_cnn_loss_grad(mx_cnn* n, const float* m, const float* h_target, int batch, float* loss_out,
@@ -839,38 +1011,39 @@ mx_status mx_cnn_loss_grad(mx_cnn* n, const float* m, const float* h_target, int
     return MX_ERR_INVALID_ARG;
   }
   cudaStream_t st = (cudaStream_t)stream;
-  MX_TRY(cnn_forward_to_pred(n, (const float4*)m, batch, st));
-  const long nc = n->cells * batch;
   const long np = num_params_total();
+  long nws = 0;
+  const WgradOuts wo = wgrad_outs(&nws);
+  float *G = n->grad, *ws = n->ws;
+  const float *P = n->params, *s = n->stats;
+  // (biases and weight sums are added to; the weights' gradient is then written whole)
   MX_CUDA_TRY(cudaMemsetAsync(n->loss, 0, sizeof(float), st));
-  MX_CUDA_TRY(cudaMemsetAsync(n->grad, 0, sizeof(float) * np, st));
-  const float* s = n->stats;
-  loss_kernel<<<(unsigned)((nc + 255) / 256), 256, 0, st>>>(
-      n->pred, (const float4*)h_target, nc, make_float3(s[6], s[7], s[8]),
-      make_float3(1.f / s[9], 1.f / s[10], 1.f / s[11]), 1.f / (3.f * (float)nc), n->dy4, n->loss);
-  MX_TRY(launch_check("loss_kernel"));
+  MX_CUDA_TRY(cudaMemsetAsync(G, 0, sizeof(float) * np, st));
+  MX_CUDA_TRY(cudaMemsetAsync(ws, 0, sizeof(float) * nws, st));
+  MX_TRY(cnn_hidden(n, (const float4*)m, batch, true, st));
   const ConvDims d = conv_dims(n, batch);
-  float* G = n->grad;
-  const unsigned bgrid = (unsigned)((nc + 1023) / 1024 < 1024 ? (nc + 1023) / 1024 : 1024);
-  // layer 4: weights, bias, then dY3 = conv(dY4, W4') * gelu'(y3)
-  MX_TRY((wgrad_run<32, 16>(n->a3, n->dy4, G + layer_w_off(3), d, 32, 3, n->flag, st)));
-  bgrad_kernel<<<bgrid, 256, 0, st>>>(n->dy4, 16, 3, nc, G + layer_w_off(3) + 3 * 32 * 27);
-  MX_TRY(launch_check("bgrad_kernel"));
-  MX_TRY((conv_run<16, 32, CM_BWD>(n->dy4, n->wb[3], nullptr, n->dy3, n->y3, nullptr, d, n->flag, st)));
-  // layer 3
-  MX_TRY((wgrad_run<64, 32>(n->a2, n->dy3, G + layer_w_off(2), d, 64, 32, n->flag, st)));
-  bgrad_kernel<<<bgrid, 256, 0, st>>>(n->dy3, 32, 32, nc, G + layer_w_off(2) + 32 * 64 * 27);
-  MX_TRY(launch_check("bgrad_kernel"));
-  MX_TRY((conv_run<32, 64, CM_BWD>(n->dy3, n->wb[2], nullptr, n->dy2, n->y2, nullptr, d, n->flag, st)));
-  // layer 2
-  MX_TRY((wgrad_run<32, 64>(n->a1, n->dy2, G + layer_w_off(1), d, 32, 64, n->flag, st)));
-  bgrad_kernel<<<bgrid, 256, 0, st>>>(n->dy2, 64, 64, nc, G + layer_w_off(1) + 64 * 32 * 27);
-  MX_TRY(launch_check("bgrad_kernel"));
-  MX_TRY((conv_run<64, 32, CM_BWD>(n->dy2, n->wb[1], nullptr, n->dy1, n->y1, nullptr, d, n->flag, st)));
-  // layer 1
-  MX_TRY((wgrad_run<16, 32>(n->x0, n->dy1, G + layer_w_off(0), d, 3, 32, n->flag, st)));
-  bgrad_kernel<<<bgrid, 256, 0, st>>>(n->dy1, 32, 32, nc, G + layer_w_off(0) + 32 * 3 * 27);
-  MX_TRY(launch_check("bgrad_kernel"));
+  auto bias = [&](float* base, int l) { return base + layer_w_off(l) + (long)kCh[l] * kCh[l + 1] * 27; };
+  ConvArgs a{};
+  a.d = d;
+  a.flag = n->flag;
+  // last layer with the loss and its gradient
+  a.wk = n->wf[3], a.bias = bias((float*)P, 3), a.out = n->dy4, a.target = (const float4*)h_target;
+  a.mean = make_float3(s[6], s[7], s[8]), a.sd = make_float3(1.f / s[9], 1.f / s[10], 1.f / s[11]);
+  a.inv_count = 1.f / (3.f * (float)(n->cells * batch)), a.loss = n->loss, a.db = bias(G, 3);
+  MX_TRY((conv_run<32, 8, CM_LOSS>(n->c_a3, a, st)));
+  // per layer: dY of the layer below (with its bias gradient), then the weight gradient
+  a.wk = n->wb[3], a.out = n->dy3, a.ypre = n->y3, a.db = bias(G, 2);
+  MX_TRY((conv_run<16, 32, CM_BWD>(n->c_dy4, a, st)));
+  MX_TRY((wgrad_run<16, 32>(n->s_dy4, n->r_a3, ws + wo.l[3].ws, d, n->flag, st)));
+  a.wk = n->wb[2], a.out = n->dy2, a.ypre = n->y2, a.db = bias(G, 1);
+  MX_TRY((conv_run<32, 64, CM_BWD>(n->c_dy3, a, st)));
+  MX_TRY((wgrad_run<32, 64>(n->s_dy3, n->r_a2, ws + wo.l[2].ws, d, n->flag, st)));
+  a.wk = n->wb[1], a.out = n->dy1, a.ypre = n->y1, a.db = bias(G, 0);
+  MX_TRY((conv_run<64, 32, CM_BWD>(n->c_dy2, a, st)));
+  MX_TRY((wgrad_run<32, 64>(n->s_a1, n->r_dy2, ws + wo.l[1].ws, d, n->flag, st)));
+  MX_TRY((wgrad_run<16, 32>(n->s_x0, n->r_dy1, ws + wo.l[0].ws, d, n->flag, st)));
+  launch_pdl(wgrad_finish_kernel, dim3((64 * 32 * 27 + 255) / 256, 4), dim3(256), 0, st, n->ws, G, wo);
+  MX_TRY(launch_check("wgrad_finish_kernel"));
   if (loss_out) MX_CUDA_TRY(cudaMemcpyAsync(loss_out, n->loss, sizeof(float), cudaMemcpyDeviceToDevice, st));
   if (grad_out) MX_CUDA_TRY(cudaMemcpyAsync(grad_out, n->grad, sizeof(float) * np, cudaMemcpyDeviceToDevice, st));
   return MX_OK;

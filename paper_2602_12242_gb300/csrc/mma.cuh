@@ -19,7 +19,8 @@ __device__ __forceinline__ float bf2f(bf16_t h) {
   return __bfloat162float(r);
 }
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
-  return (uint32_t)f2bf(a) | ((uint32_t)f2bf(b) << 16);
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);  // one conversion for both
+  return *reinterpret_cast<const uint32_t*>(&v);
 }
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 

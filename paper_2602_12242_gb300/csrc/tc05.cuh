@@ -69,6 +69,28 @@ __device__ __forceinline__ void tc_mma_bf16(uint32_t dtmem, uint64_t adesc, uint
       : "memory");
 }
 
+// The same with the descriptors' low words given (start address and LBO; an
+// operand further along in the same layout is an addition of bytes / 16 to it).
+// Executed by a converged warp; the thread with `leader` set issues.
+__device__ __forceinline__ void tc_mma_bf16_lo(uint32_t dtmem, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
+                                               uint32_t idesc, bool accumulate, uint32_t leader) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
+      "setp.ne.b32 p, %6, 0;\n\t"
+      "setp.ne.b32 q, %7, 0;\n\t"
+      "mov.b64 a, {%1, %2};\n\t"
+      "mov.b64 b, {%3, %4};\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}" ::"r"(dtmem),
+      "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"((uint32_t)accumulate), "r"(leader)
+      : "memory");
+}
+// 1 in one thread of the converged warp
+__device__ __forceinline__ uint32_t tc_elect() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r;
+}
+
 // Arrive on the mbarrier once every MMA issued so far by this thread is complete.
 __device__ __forceinline__ void tc_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tc_smem_addr(bar))

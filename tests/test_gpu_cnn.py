@@ -164,3 +164,31 @@ def test_trained_surrogate_gain_against_fft():
           f"surrogate {1e3 * bat['surrogate']:.1f} us")
     assert err < 0.25 and err < 0.5 * err0, (err, err0)
     assert bat["surrogate"] < bat["fft"], bat
+
+
+@pytest.mark.parametrize("shape,batch", [((1, 1, 1), 1), ((1, 33, 17), 3), ((2, 16, 8), 1), ((5, 9, 20), 2),
+                                         ((2, 17, 33), 60), ((7, 8, 16), 40), ((3, 40, 9), 21)])
+def test_tile_walk_matches_oracle(shape, batch):
+    """Grids of less than a tile, tiles cut at every edge, one to seven layers, and batches whose
+    tile ranges start inside a column: forward, loss and every parameter block's gradient, at
+    the tolerances of the tests above."""
+    net, flat = _net(shape, batch, seed=61)
+    net.set_normalizer(STATS)
+    m = _fields(shape, batch, 62).astype(np.float32).astype(np.float64)
+    h = net.forward(_dev(m))[..., :3].double().cpu().numpy().reshape((batch,) + shape + (3,))
+    assert rel_l2(h, _oracle_forward(flat, m, STATS)) <= 1e-3
+    rng = np.random.default_rng(63)
+    tgt = (np.array(STATS[6:9]) + np.array(STATS[9:12]) * rng.normal(size=(batch,) + shape + (3,)))
+    tgt = tgt.astype(np.float32).astype(np.float64)
+    mean_in, std_in = np.array(STATS[0:3], np.float32), np.array(STATS[3:6], np.float32)
+    x = ocnn.to_ncdhw(torch.as_tensor(((m - mean_in) / std_in).astype(np.float32), dtype=torch.float64))
+    t = ocnn.to_ncdhw((tgt - np.array(STATS[6:9])) / np.array(STATS[9:12]))
+    L_ref, g_ref = ocnn.loss_and_grad(torch.as_tensor(flat), x, t, rnd=ocnn.bf16_round)
+    for _ in range(2):  # (again on the same buffers: nothing of the first pass is left in them)
+        loss, grad = net.loss_grad(_dev(m), _dev(tgt))
+        assert abs(float(loss) - L_ref) <= 1e-3 * abs(L_ref)
+        g, o = grad.double().cpu().numpy(), 0
+        for s in ocnn.param_shapes():
+            n = int(np.prod(s))
+            assert rel_l2(g[o:o + n], g_ref.numpy()[o:o + n]) <= 3e-2, s
+            o += n
