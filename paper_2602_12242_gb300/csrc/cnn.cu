@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(ConvTc<CIN, COUT>::threads, 1)
     if (lane < 27)
       bulk_load(smraw + lane * (T::w_bytes / 27), p.wk + (long)lane * (T::w_bytes / 27 / sizeof(bf16_t)),
                 T::w_bytes / 27, &wbar);
-    pdl_wait();
+    pdl_wait_next();
     if (lane == 0) {
       int seq = 0;
       bool ok = true;
@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(ConvTc<CIN, COUT>::threads, 1)
     const int row = 32 * (warp & 3) + lane;
     const int cx = row & 7, cy = row >> 3;
     const int cb = (warp - 2) / 4 * NH;
-    pdl_wait();
+    pdl_wait_next();
     float bv[NH];
 #pragma unroll
     for (int c = 0; c < NH; ++c) bv[c] = (MODE == CM_BWD || cb + c >= COUT || (COUT == 8 && cb + c >= 3)) ? 0.f : __ldg(&p.bias[cb + c]);
@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(192, 2)
     const int zp = bz % d.nz + dz - 1;
     return zp >= 0 && zp < d.nz;
   };
-  pdl_wait();
+  pdl_wait_next();
   if (warp == 0) {
     if (lane == 0) {
       int k = 0;
@@ -542,7 +542,7 @@ struct WgradOuts {
 };
 __global__ void wgrad_finish_kernel(const float* __restrict__ ws, float* __restrict__ grad, WgradOuts o) {
   const WgradOut l = o.l[blockIdx.y];
-  pdl_wait();
+  pdl_wait_next();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= l.cout * l.cin * 27) return;
   const int tap = e % 27, ci = e / 27 % l.cin, co = e / 27 / l.cin;
@@ -556,7 +556,7 @@ __global__ void wgrad_finish_kernel(const float* __restrict__ ws, float* __restr
 __global__ void normalize_in_kernel(const float4* __restrict__ m, bf16_t* __restrict__ x0, ConvDims d, long ncells,
                                     float3 mean, float3 inv_std) {
   const long c = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  pdl_wait();
+  pdl_wait_next();
   if (c >= ncells) return;
   const float4 v = m[c];
   const int x = (int)(c % d.nx), y = (int)(c / d.nx % d.ny);

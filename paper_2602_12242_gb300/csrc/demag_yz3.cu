@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(NT, NT == 512 && E <= 16 && P <= 8 ? 2 : 1) yz
 #pragma unroll
     for (int q = 0; q < NE; ++q) pre[q] = z_entry(k.tq, qzs, min(2 * q + mypar, P / 2));
   }
-  pdl_wait();  // w1 is the previous kernel's
+  pdl_wait_next();  // w1 is the previous kernel's
   __syncthreads();  // the twiddle tables
   {
     const int total = nlines * LH;

@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(SMALL ? 384 : 128)
   const long r = blockIdx.x;
   float* row = v + r * kFC * Wp;
   if (SMALL) fno_stage_tw(ts, tw, Wp, P, K);
-  pdl_wait();
+  pdl_wait_next();
   if (LIFT) {
     // a thread takes one cell and eight channels
     for (int q = threadIdx.x; q < Wp * 4; q += blockDim.x) {
@@ -256,7 +256,7 @@ __global__ void __cluster_dims__(kMidCl, 1, 1) __launch_bounds__(kMidWarps * 32)
   const bool ti = HH * M2 <= kMidTi;
   if (ti)
     for (int q = threadIdx.x; q < (ye - yb) * M2; q += blockDim.x) s.ti[q] = __ldg(&twy[(long)yb * M2 + q]);
-  pdl_wait();
+  pdl_wait_next();
   // warp -> (mode of this CTA, share of the sum)
   const int ns = fno_mid_shares(K), mj = warp % MM, sp = warp / MM;
   const bool sums = sp < ns && mj < nm;
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(128) fno_dft_y_kernel(const float2* __restrict
         __syncthreads();
         for (int q = threadIdx.x; q < ny * kMidM; q += 128)
           ts[q / kMidM][q % kMidM] = __ldg(&twy[(long)(yc + q / kMidM) * M2 + min(m0 + q % kMidM, M2 - 1)]);
-        if (sp == 0 && yc == 0) pdl_wait();
+        if (sp == 0 && yc == 0) pdl_wait_next();
         __syncthreads();
       }
       for (int y0 = sp; y0 < ny; y0 += 8 * ns) {
@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(256) fno_mix_kernel(const float2* __restrict__
     else
       F[i][o] = r;
   }
-  pdl_wait();
+  pdl_wait_next();
   const int o = threadIdx.x & 31, w = threadIdx.x >> 5;
   const float2* Xm = X + (long)mode * B * kFC;
   float2* Ym = Y + (long)mode * B * kFC;
@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(128) fno_idft_y_kernel(const float2* __restric
   const int b = ok ? (int)(col / K) : 0, kx = (int)(col % K);
   for (int q = threadIdx.x; q < M2 * kMidY; q += 128)
     ts[q % M2][q / M2] = __ldg(&twy[(long)min(y0 + q / M2, H - 1) * M2 + q % M2]);
-  pdl_wait();
+  pdl_wait_next();
   __syncthreads();
   if (!ok) return;
   const float2* v = Y + ((long)kx * B + b) * kFC + o;
@@ -545,7 +545,7 @@ __global__ void __launch_bounds__(T == 8 ? 256 : 512, T == 8 ? 2 : 1)
   float bias[T];
 #pragma unroll
   for (int j = 0; j < T; ++j) bias[j] = (!BWD && wl) ? __ldg(&wl[j / 4 * 16 + 4 * og + j % 4]) : 0.f;
-  pdl_wait();
+  pdl_wait_next();
   fno_copy_row(vs, vin + base, Wp, P);
   float2* Ar = A + r * K * kFC;
   for (int q = tid; q < K * kFC; q += NT) {
@@ -704,7 +704,7 @@ __global__ void __launch_bounds__(kPN) fno_proj_kernel(const float* __restrict__
   __shared__ __align__(16) float Q1t[kFC * (kFH + 4)], q1s[kFH], Q2s[3 * kFH], vs[kFC * kPP];
   __shared__ float red[8][3][kPT];
   fno_proj_weights(Q1t, q1s, Q2s, Q1, q1, Q2);
-  pdl_wait();
+  pdl_wait_next();
   fno_load_tile(vs, v, blockIdx.x, groups, Wp);
   __syncthreads();
   const int tid = threadIdx.x, xg = tid & 7, jg = tid >> 3;
@@ -766,7 +766,7 @@ __global__ void __launch_bounds__(kPN, 2)
   FnoTrainSmem& s = *reinterpret_cast<FnoTrainSmem*>(trraw);
   const int tid = threadIdx.x, xg = tid & 7, jg = tid >> 3, lane = tid & 31, warp = tid >> 5;
   fno_proj_weights(s.Q1t, s.q1s, s.Q2s, Q1, q1, Q2);
-  pdl_wait();
+  pdl_wait_next();
   const long ntiles = (groups + kPT / 4 - 1) / (kPT / 4);
   // dQ1[jr + 16 a][ir + 8 b] over half kh of the tile's cells
   const int jr = tid & 15, ir = (tid >> 4) & 7, kh = tid >> 7;
@@ -947,7 +947,7 @@ __global__ void __launch_bounds__(256) fno_wgrad_kernel(const float* __restrict_
   float* bs = as + kFC * kWgP;
   const int tid = threadIdx.x, o0 = tid & 7, i0 = (tid >> 3) & 7, grp = tid >> 6;
   float acc[4][4] = {}, ab[4] = {};
-  pdl_wait();
+  pdl_wait_next();
   const int per = (Wp + kWgX - 1) / kWgX;
   // the next chunk's loads are in flight while this one is summed
   constexpr int NL = kFC * (kWgX / 4) / 256;
@@ -1015,7 +1015,7 @@ __global__ void __launch_bounds__(1024) fno_lift_grad_kernel(const float* __rest
                                                              float* __restrict__ dP, float* __restrict__ dp) {
   const int o = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float a[4] = {};
-  pdl_wait();
+  pdl_wait_next();
   for (long r = blockIdx.x; r < rows; r += gridDim.x) {
     const float* d = du + (r * kFC + o) * Wp;
     for (int x = lane; x < W; x += 32) {
@@ -1043,7 +1043,7 @@ __global__ void __launch_bounds__(1024) fno_rgrad_kernel(const float2* __restric
   __shared__ float2 xs[kFC][kFC];
   __shared__ float2 gs[kFC][kFC];
   const int mode = blockIdx.x, kx = mode % K;
-  pdl_wait();
+  pdl_wait_next();
   const int i = threadIdx.x >> 5, o = threadIdx.x & 31;
   const float2* Xm = X + (long)mode * B * kFC;
   const float2* Gm = Xg + (long)mode * B * kFC;
