@@ -70,14 +70,30 @@ constexpr double kAdjStoreBytes = 4.0e9;
 // prep: for state m (stencil), its demag field hd and the cotangent v of
 // its stage rate, g_m = c [H x v + alpha (v (m.H) + H (v.m) - 2 m (v.H))] and
 // w = g_H / Ms with g_H = c [v x m + alpha (m (v.m) - v |m|^2)].
+// What prep reads, held.
+struct PrepIn {
+  float3 m, hd, e;
+  float ms, cK;
+  Nbrs b;
+  __device__ __forceinline__ void load(const float4* __restrict__ mf, const float4* __restrict__ hdf, const Grid& g,
+                                       const LocalCoef& c, int i, int j, int k, long idx) {
+    m = f3(mf[idx]);
+    hd = hdf ? f3(__ldg(&hdf[idx])) : make_float3(0.f, 0.f, 0.f);
+    e = easy_axis(c, idx);
+    ms = c.ms_map ? __ldg(&c.ms_map[idx]) : c.Ms;
+    cK = aniso_coef(c, idx);
+    neighbours(mf, g, c, i, j, k, idx, m, b.xp, b.xm, b.yp, b.ym, b.zp, b.zm);
+  }
+};
+
+// prep from held inputs; writes w and g_m and returns w
 template <bool DMI>
-__device__ __forceinline__ void prep_cell(const float4* __restrict__ m, const float4* __restrict__ hd, const Grid& g,
-                                          const LocalCoef& c, int i, int j, int k, long idx, float3 v,
-                                          float4* __restrict__ wbuf, float4* __restrict__ gm) {
-  const float3 mc = f3(m[idx]);
-  const float ms = c.ms_map ? __ldg(&c.ms_map[idx]) : c.Ms;
+__device__ __forceinline__ float3 prep_apply(const PrepIn& in, const LocalCoef& c, long idx, float3 v,
+                                             float4* __restrict__ wbuf, float4* __restrict__ gm) {
+  const float3 mc = in.m;
+  const float ms = in.ms;
   Terms t;
-  local_terms<DMI>(m, hd, g, c, i, j, k, idx, mc, 1.f / ms, t);
+  local_terms_nb<DMI>(in.b, in.hd, c, mc, 1.f / ms, in.e, in.cK, t);
   const float3 H = t.demag + t.exch + t.anis + t.dmi + t.zee;
   const float mH = dot3(mc, H), vm = dot3(v, mc), vH = dot3(v, H), mm = dot3(mc, mc);
   float3 gmv = c.alpha * (mH * v + vm * H - (2.f * vH) * mc);
@@ -90,60 +106,93 @@ __device__ __forceinline__ void prep_cell(const float4* __restrict__ m, const fl
   gh = (c.llg / ms) * gh;
   gm[idx] = make_float4(gmv.x, gmv.y, gmv.z, 0.f);
   wbuf[idx] = make_float4(gh.x, gh.y, gh.z, 0.f);
+  return gh;
+}
+
+template <bool DMI>
+__device__ __forceinline__ void prep_cell(const float4* __restrict__ m, const float4* __restrict__ hd, const Grid& g,
+                                          const LocalCoef& c, int i, int j, int k, long idx, float3 v,
+                                          float4* __restrict__ wbuf, float4* __restrict__ gm) {
+  PrepIn in;
+  in.load(m, hd, g, c, i, j, k, idx);
+  prep_apply<DMI>(in, c, idx, v, wbuf, gm);
 }
 
 // finish: lam_m = g_m + Ms (L w) (w's stencil and hdw, the demag field of
 // w); the Ms gradient term; the stage's share of lam_acc; returns the next
 // stage rate's cotangent (STAGE 3, 2, 1) or zero (STAGE 0).
-template <bool DMI, int STAGE>
-__device__ __forceinline__ float3 finish_cell_v(const float4* __restrict__ m, const float4* __restrict__ wbuf,
-                                                float3 hdwv, const float4* __restrict__ gm,
-                                                const float4* __restrict__ lam_u4, float4* __restrict__ lam_acc,
-                                                double* __restrict__ dms, const Grid& g, const LocalCoef& c, float dt,
-                                                int i, int j, int k, long idx) {
-  const float ms = c.ms_map ? __ldg(&c.ms_map[idx]) : c.Ms;
-  const float inv_ms = 1.f / ms;
+// What finish reads, held (stage: 3, 2, 1 or 0).
+struct FinishIn {
+  float3 w, gm, u4, e;
+  float4 m4, lam;
+  float ms, cK;
+  double dm;
+  Nbrs bw, bm;
+  __device__ __forceinline__ void load(const float4* __restrict__ mf, const float4* __restrict__ wbuf,
+                                       const float4* __restrict__ gmf, const float4* __restrict__ lam_u4,
+                                       const float4* __restrict__ lam_acc, const double* __restrict__ dms,
+                                       const Grid& g, const LocalCoef& c, int i, int j, int k, long idx, int stage) {
+    w = f3(wbuf[idx]);
+    m4 = mf[idx];
+    gm = f3(gmf[idx]);
+    lam = lam_acc[idx];
+    u4 = stage > 0 ? f3(lam_u4[idx]) : make_float3(0.f, 0.f, 0.f);
+    e = easy_axis(c, idx);
+    ms = c.ms_map ? __ldg(&c.ms_map[idx]) : c.Ms;
+    cK = aniso_coef(c, idx);
+    neighbours(wbuf, g, c, i, j, k, idx, w, bw.xp, bw.xm, bw.yp, bw.ym, bw.zp, bw.zm);
+    dm = 0.0;
+    if (dms) {
+      dm = dms[idx];
+      neighbours(mf, g, c, i, j, k, idx, f3(m4), bm.xp, bm.xm, bm.yp, bm.ym, bm.zp, bm.zm);
+    }
+  }
+};
+
+template <bool DMI>
+__device__ __forceinline__ float3 finish_apply(const FinishIn& in, float3 hdwv, float4* __restrict__ lam_acc,
+                                               double* __restrict__ dms, const LocalCoef& c, float dt, long idx,
+                                               int stage) {
+  const float ms = in.ms, inv_ms = 1.f / ms;
   // L applied to w = g_H / Ms: demag from the convolution, local terms here
   LocalCoef cl = c;
   cl.hx = cl.hy = cl.hz = 0.f;  // the bias is not part of the linear operator
-  const float3 wc = f3(wbuf[idx]);
+  const float3 wc = in.w;
   Terms tw;
-  local_terms_v<DMI>(wbuf, hdwv, g, cl, i, j, k, idx, wc, inv_ms, tw);
+  local_terms_nb<DMI>(in.bw, hdwv, cl, wc, inv_ms, in.e, in.cK, tw);
   const float3 Lw = tw.demag + tw.exch + tw.anis + tw.dmi;
-  const float4 m4 = m[idx];
-  const float3 mc = f3(m4);
-  const float3 lam_m = f3(gm[idx]) + ms * Lw;
+  const float3 mc = f3(in.m4);
+  const float3 lam_m = in.gm + ms * Lw;
   // Ms gradient: m . (demag of g_H) - w . (L_local m)
   if (dms) {
     Terms tm;
-    local_terms<DMI>(m, nullptr, g, cl, i, j, k, idx, mc, inv_ms, tm);
+    local_terms_nb<DMI>(in.bm, make_float3(0.f, 0.f, 0.f), cl, mc, inv_ms, in.e, in.cK, tm);
     const float3 Lm = tm.exch + tm.anis + tm.dmi;
-    dms[idx] += (double)dot3(mc, tw.demag) - (double)dot3(wc, Lm);
+    dms[idx] = in.dm + ((double)dot3(mc, tw.demag) - (double)dot3(wc, Lm));
   }
-  if (STAGE == 0) {
-    const float4 a = lam_acc[idx];
+  const float4 a = in.lam;
+  if (stage == 0) {
     lam_acc[idx] = make_float4(a.x + lam_m.x, a.y + lam_m.y, a.z + lam_m.z, 0.f);
     return make_float3(0.f, 0.f, 0.f);
   }
   // J_N(u_s)^T lam_m with n = m (unit), |u_s| in m.w
-  const float3 lu = (1.f / m4.w) * (lam_m - dot3(mc, lam_m) * mc);
-  const float4 a = lam_acc[idx];
+  const float3 lu = (1.f / in.m4.w) * (lam_m - dot3(mc, lam_m) * mc);
   lam_acc[idx] = make_float4(a.x + lu.x, a.y + lu.y, a.z + lu.z, 0.f);
-  const float3 u4 = f3(lam_u4[idx]);
-  const float cu4 = (STAGE == 1) ? dt / 6.f : dt / 3.f;
-  const float cus = (STAGE == 3) ? dt : 0.5f * dt;
-  return cu4 * u4 + cus * lu;
+  const float cu4 = (stage == 1) ? dt / 6.f : dt / 3.f;
+  const float cus = (stage == 3) ? dt : 0.5f * dt;
+  return cu4 * in.u4 + cus * lu;
 }
 
-// The same with the demag field of w read from hdw (zero if hdw is null).
+// finish with the demag field of w read from hdw (zero if hdw is null).
 template <bool DMI, int STAGE>
 __device__ __forceinline__ float3 finish_cell(const float4* __restrict__ m, const float4* __restrict__ wbuf,
                                               const float4* __restrict__ hdw, const float4* __restrict__ gm,
                                               const float4* __restrict__ lam_u4, float4* __restrict__ lam_acc,
                                               double* __restrict__ dms, const Grid& g, const LocalCoef& c, float dt,
                                               int i, int j, int k, long idx) {
-  return finish_cell_v<DMI, STAGE>(m, wbuf, hdw ? f3(__ldg(&hdw[idx])) : make_float3(0.f, 0.f, 0.f), gm, lam_u4,
-                                   lam_acc, dms, g, c, dt, i, j, k, idx);
+  FinishIn in;
+  in.load(m, wbuf, gm, lam_u4, lam_acc, dms, g, c, i, j, k, idx, STAGE);
+  return finish_apply<DMI>(in, hdw ? f3(__ldg(&hdw[idx])) : make_float3(0.f, 0.f, 0.f), lam_acc, dms, c, dt, idx, STAGE);
 }
 
 template <bool DMI>
@@ -240,87 +289,79 @@ struct AdjRowArgs {
 };
 
 // begin of a reverse step at one cell (lam_u4 = J_N(u4)^T lam_acc with u4's
-// norm in mnew.w, lam_acc = lam_u4) and the prep of its last stage
+// norm in mnew.w, lam_acc = lam_u4) and the prep of its last stage; returns its w
 template <bool DMI>
-__device__ __forceinline__ void adj_begin_cell(const AdjRowArgs& a, const float4* __restrict__ mnew, const Grid& g,
-                                               const LocalCoef& c, float dt, int i, int y, int z, long idx) {
-  const float4 n4 = mnew[idx];
+__device__ __forceinline__ float3 adj_begin_cell(const AdjRowArgs& a, float4 n4, float3 l, const PrepIn& in,
+                                                 const LocalCoef& c, float dt, long idx) {
   const float3 nc = f3(n4);
-  const float3 l = f3(a.lam_acc[idx]);
   const float3 lu = (1.f / n4.w) * (l - dot3(nc, l) * nc);
   a.lam_u4[idx] = make_float4(lu.x, lu.y, lu.z, 0.f);
   a.lam_acc[idx] = make_float4(lu.x, lu.y, lu.z, 0.f);
-  prep_cell<DMI>(a.m_prev, a.hd_prev, g, c, i, y, z, idx, (dt / 6.f) * lu, a.wbuf_out, a.gm_out);
+  return prep_apply<DMI>(in, c, idx, (dt / 6.f) * lu, a.wbuf_out, a.gm_out);
 }
 
-template <bool DMI, int R, int NT>
-__device__ __forceinline__ void adj_row_begin_cells(const AdjRowArgs& a, const Grid& g, const LocalCoef& c, float dt,
-                                                    int row0) {
-  const int total = min(R, g.ny * g.nz - row0) * g.nx;
-  for (int e = threadIdx.x; e < total; e += NT) {
-    const int r = e / g.nx, i = e - r * g.nx;
-    const int row = row0 + r;
-    const int z = row / g.ny, y = row - z * g.ny;
-    adj_begin_cell<DMI>(a, a.mnew, g, c, dt, i, y, z, (long)row * g.nx + i);
-  }
-}
-
-// STAGE 0 with CHAIN: after the finish, the begin of the step before at the
-// same cell (its result is this step's start state a.m) with the prep of its
-// last stage (a.m_prev, a.hd_prev -> a.wbuf_out, a.gm_out).
-template <bool DMI, int STAGE, int E, int S, int R, int NT, bool CHAIN = false>
-__device__ __forceinline__ void adj_row_cells(const float2* sm, const AdjRowArgs& a, const Grid& g,
-                                              const LocalCoef& c, float dt, int row0) {
-  const int total = min(R, g.ny * g.nz - row0) * g.nx;
-  for (int e = threadIdx.x; e < total; e += NT) {
-    const int r = e / g.nx, i = e - r * g.nx;
-    const int row = row0 + r;
-    const int z = row / g.ny, y = row - z * g.ny;
-    const long idx = (long)row * g.nx + i;
-    const float3 nk = finish_cell_v<DMI, STAGE>(a.m, a.wbuf, xi_cell<E, S>(sm, r, i), a.gm, a.lam_u4, a.lam_acc,
-                                                a.dms, g, c, dt, i, y, z, idx);
-    if (STAGE > 0) prep_cell<DMI>(a.m_prev, a.hd_prev, g, c, i, y, z, idx, nk, a.wbuf_out, a.gm_out);
-    if (STAGE == 0 && CHAIN) adj_begin_cell<DMI>(a, a.m, g, c, dt, i, y, z, idx);
-  }
-}
-
-template <int E, int S, int R, int NT, bool DMI>
-__global__ void __launch_bounds__(NT) adj_row_begin_kernel(float2* __restrict__ w1, Grid g, float ms,
-                                                           const float* __restrict__ ms_map,
+template <int M, int R, int NT, bool DMI>
+__global__ void __launch_bounds__(NT) adj_row_begin_kernel(float2* __restrict__ w1, Grid g,
                                                            const float2* __restrict__ twM,
                                                            const float2* __restrict__ twP, AdjRowArgs a, LocalCoef c,
                                                            float dt) {
   extern __shared__ float2 sm[];
   const int row0 = blockIdx.x * R;
-  pdl_wait();
-  adj_row_begin_cells<DMI, R, NT>(a, g, c, dt, row0);
-  __syncthreads();
-  xf_rows<E, S, R, NT, true>(sm, a.wbuf_out, g, ms, ms_map, w1, row0, twM, twP);
+  RowTw<M> tw;
+  tw.load(twM, twP);
+  pdl_wait_next();
+  const int total = min(R, g.ny * g.nz - row0) * g.nx;
+  for (int e = threadIdx.x; e < total; e += NT) {
+    const int r = R == 1 ? 0 : e / g.nx, i = e - r * g.nx;
+    const int row = row0 + r;
+    const long idx = (long)row0 * g.nx + e;
+    PrepIn in;
+    in.load(a.m_prev, a.hd_prev, g, c, i, row % g.ny, row / g.ny, idx);
+    const float3 w = adj_begin_cell<DMI>(a, a.mnew[idx], f3(a.lam_acc[idx]), in, c, dt, idx);
+    xf_cell<M, R>(sm, r, i, in.ms * w);
+  }
+  xf_rows<M, R>(sm, g, w1, row0, tw);
 }
 
-template <int E, int S, int R, int NT, bool DMI>
-__global__ void __launch_bounds__(NT) adj_row_kernel(float2* __restrict__ w1, Grid g, float ms,
-                                                     const float* __restrict__ ms_map, const float2* __restrict__ twM,
+// chain (stage 0): after the finish, the begin of the step before at the same
+// cell (its result is this step's start state a.m) with the prep of its last
+// stage (a.m_prev, a.hd_prev -> a.wbuf_out, a.gm_out).  What a cell of the block's
+// first NT reads is loaded before the transforms.
+template <int M, int R, int NT, bool DMI>
+__global__ void __launch_bounds__(NT) adj_row_kernel(float2* __restrict__ w1, Grid g, const float2* __restrict__ twM,
                                                      const float2* __restrict__ twP, AdjRowArgs a, LocalCoef c,
                                                      float dt, int stage, int chain) {
   extern __shared__ float2 sm[];
   const int row0 = blockIdx.x * R;
-  pdl_wait();
-  xi_rows<E, S, R, NT>(sm, w1, g, row0, twM, twP);
-  switch (stage) {
-    case 3: adj_row_cells<DMI, 3, E, S, R, NT>(sm, a, g, c, dt, row0); break;
-    case 2: adj_row_cells<DMI, 2, E, S, R, NT>(sm, a, g, c, dt, row0); break;
-    case 1: adj_row_cells<DMI, 1, E, S, R, NT>(sm, a, g, c, dt, row0); break;
-    default:
-      if (!chain) {
-        adj_row_cells<DMI, 0, E, S, R, NT>(sm, a, g, c, dt, row0);
-        return;
-      }
-      adj_row_cells<DMI, 0, E, S, R, NT, true>(sm, a, g, c, dt, row0);
-      break;
+  RowTw<M> tw;
+  tw.load(twM, twP);
+  const int total = min(R, g.ny * g.nz - row0) * g.nx;
+  const bool next = stage > 0 || chain;
+  pdl_wait_next();
+  FinishIn fin;
+  PrepIn pin;
+  auto load = [&](int e) {
+    const int r = R == 1 ? 0 : e / g.nx, i = e - r * g.nx;
+    const int row = row0 + r;
+    const int z = row / g.ny, y = row - z * g.ny;
+    const long idx = (long)row0 * g.nx + e;
+    fin.load(a.m, a.wbuf, a.gm, a.lam_u4, a.lam_acc, a.dms, g, c, i, y, z, idx, stage);
+    if (next) pin.load(a.m_prev, a.hd_prev, g, c, i, y, z, idx);
+  };
+  if ((int)threadIdx.x < total) load(threadIdx.x);
+  xi_rows<M, R>(sm, w1, g, row0, tw);
+#pragma unroll 1
+  for (int e = threadIdx.x; e < total; e += NT) {
+    if (e >= NT) load(e);
+    const int r = R == 1 ? 0 : e / g.nx, i = e - r * g.nx;
+    const long idx = (long)row0 * g.nx + e;
+    const float3 nk = finish_apply<DMI>(fin, xi_cell<M, R>(sm, r, i), a.lam_acc, a.dms, c, dt, idx, stage);
+    if (!next) continue;
+    const float3 w = stage > 0 ? prep_apply<DMI>(pin, c, idx, nk, a.wbuf_out, a.gm_out)
+                               : adj_begin_cell<DMI>(a, fin.m4, f3(a.lam_acc[idx]), pin, c, dt, idx);
+    xf_cell<M, R>(sm, r, i, pin.ms * w);
   }
-  __syncthreads();  // the block's rows of the new w are written; the c2r lines are read
-  xf_rows<E, S, R, NT, true>(sm, a.wbuf_out, g, ms, ms_map, w1, row0, twM, twP);
+  if (next) xf_rows<M, R>(sm, g, w1, row0, tw);
 }
 
 // Launches the begin kernel (begin) or the stage kernel of `stage` for the
@@ -333,22 +374,20 @@ struct AdjRowLaunch {
   bool begin;
   bool chain;
   cudaStream_t st;
-  template <int E, int S, int R, int NT> mx_status run() {
-    const size_t sm = sizeof(float2) * XfShape<S, R>::lines * LineFft<E, S>::kPitch;
-    static_assert(sizeof(float2) * XfShape<S, R>::lines * LineFft<E, S>::kPitch <= 48 * 1024,
-                  "row kernel shared memory");
+  template <int M, int R, int NT> mx_status run() {
     const Grid& g = ctx->g;
     const LocalCoef c = local_coef(ctx);
     const dim3 grid((g.ny * g.nz + R - 1) / R);
     if (begin) {
-      auto k = c.dmi ? adj_row_begin_kernel<E, S, R, NT, true> : adj_row_begin_kernel<E, S, R, NT, false>;
-      launch_pdl(k, grid, dim3(NT), sm, st, ctx->w1, g, (float)ctx->p.Ms, ctx->ms_map, ctx->tw_m, ctx->tw_x, *a,
-                 c, dt);
+      auto k = c.dmi ? adj_row_begin_kernel<M, R, NT, true> : adj_row_begin_kernel<M, R, NT, false>;
+      RowShape<M, R>::allow(k);
+      launch_pdl(k, grid, dim3(NT), RowShape<M, R>::smem, st, ctx->w1, g, ctx->tw_m, ctx->tw_x, *a, c, dt);
       return launch_check("adj_row_begin_kernel");
     }
-    auto k = c.dmi ? adj_row_kernel<E, S, R, NT, true> : adj_row_kernel<E, S, R, NT, false>;
-    launch_pdl(k, grid, dim3(NT), sm, st, ctx->w1, g, (float)ctx->p.Ms, ctx->ms_map, ctx->tw_m, ctx->tw_x, *a, c,
-               dt, stage, chain ? 1 : 0);
+    auto k = c.dmi ? adj_row_kernel<M, R, NT, true> : adj_row_kernel<M, R, NT, false>;
+    RowShape<M, R>::allow(k);
+    launch_pdl(k, grid, dim3(NT), RowShape<M, R>::smem, st, ctx->w1, g, ctx->tw_m, ctx->tw_x, *a, c, dt, stage,
+               chain ? 1 : 0);
     return launch_check("adj_row_kernel");
   }
 };

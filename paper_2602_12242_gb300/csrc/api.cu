@@ -107,10 +107,11 @@ static std::vector<float2> twiddles32(int L) {
   return t;
 }
 
-// Whether an RK4 step runs as y/z passes plus one row kernel per stage.
-bool row_steps(const mx_ctx* ctx, int method) {
-  return method == MX_RK4 && ctx->p.demag && ctx->xrow && !ctx->plane && !ctx->surrogate && !ctx->fno;
-}
+// Whether the inverse x pass and the local stage are one row kernel.
+static bool row_kernels(const mx_ctx* ctx) { return ctx->xrow && !ctx->plane && !ctx->surrogate && !ctx->fno; }
+
+// Whether an RK4 or Euler step runs as y/z passes plus one row kernel per stage.
+bool row_steps(const mx_ctx* ctx, int method) { return method != MX_MRI && ctx->p.demag && row_kernels(ctx); }
 
 // The forward x pass of m into w1, which the first row-kernel step of a
 // sequence needs (each later step finds it left by the step before).
@@ -131,7 +132,12 @@ static mx_status enqueue_step(mx_ctx* ctx, float4* m, double dt, int method, cud
   const bool xlocal = demag && ctx->xlocal;
   if (method == MX_EULER) {
     StageIO io{m, hd, m, ctx->acc, ctx->sa, (float)dt, MX_TERM_ALL};
-    if (xlocal) {
+    if (row_steps(ctx, method)) {
+      if (lead) MX_TRY(lead_x_pass(ctx, m, st));
+      MX_TRY(demag_yz(ctx, st));
+      ProfScope ps(ctx, KID_X_INV_LOCAL, st);
+      MX_TRY(fast_row_stage(ctx, LM_EULER, io, tail, nullptr, st));
+    } else if (xlocal) {
       MX_TRY(plane_stage_xlocal(ctx, LM_EULER, io, st));
     } else {
       if (demag) MX_TRY(demag_field(ctx, m, hd, st));
@@ -214,7 +220,7 @@ const char* mx_kernel_name(const mx_ctx* ctx, int q) {
     case KID_YZ:
       if (ctx->yz3) return "yz3_kernel";
       if (ctx->plane) return ctx->quad ? "yzq_kernel" : "yzh_kernel";
-      return ctx->yz2d ? "yz2d_kernel" : "yz_fused_kernel";
+      return ctx->yz2d ? (yz2d_wide(ctx->g) ? "yz2d_wide_kernel" : "yz2d_kernel") : "yz_fused_kernel";
     case KID_Y_FWD: return ctx->deep ? "deep_yf_kernel" : "y_fwd_kernel";
     case KID_Z_MUL: return ctx->deep ? (ctx->g.Pz > 128 ? "deep_z3_kernel" : "deep_z_kernel") : "z_mul_kernel";
     case KID_Y_INV: return ctx->deep ? "deep_yi_kernel" : "y_inv_kernel";
@@ -453,8 +459,15 @@ mx_status mx_heff(mx_ctx* ctx, const float* m, float* h, int terms, mx_stream_t 
     set_error("mx_heff: demag kernel not built");
     return MX_ERR_NOT_BUILT;
   }
-  if (demag) MX_TRY(demag_field(ctx, (const float4*)m, ctx->hd, st));
   StageIO io{(const float4*)m, demag ? ctx->hd : nullptr, nullptr, nullptr, (float4*)h, 0.f, terms};
+  if (demag && row_kernels(ctx)) {
+    // three launches (forward x, y/z, row kernel), not four
+    MX_TRY(lead_x_pass(ctx, io.m, st));
+    MX_TRY(demag_yz(ctx, st));
+    ProfScope ps(ctx, KID_X_INV_LOCAL, st);
+    return fast_row_stage(ctx, LM_HEFF, io, false, nullptr, st);
+  }
+  if (demag) MX_TRY(demag_field(ctx, io.m, ctx->hd, st));
   return local_stage(ctx, LM_HEFF, io, st);
 }
 

@@ -64,11 +64,14 @@ struct StageIO;
 mx_status plane_stage_xlocal(mx_ctx* ctx, int mode, const StageIO& io, cudaStream_t st);
 // The y/z passes of demag_field alone (w1 in place, after the forward x pass).
 mx_status demag_yz(mx_ctx* ctx, cudaStream_t st);
-// One RK4 stage's row kernel on grids with ctx->xrow (demag_fast.cu): the
-// inverse x pass of w1, the local stage of `mode` (with hd_out, the demag
-// field of io.m is also written there), and with xf_next the forward x pass
-// of io.out into w1 for the next stage.
+// The row kernel of an RK4 stage or an Euler step on grids with ctx->xrow
+// (demag_fast.cu): the inverse x pass of w1, the local stage of `mode` (with
+// hd_out, the demag field of io.m is also written there), and with xf_next the
+// forward x pass of io.out into w1 for the next stage.  With LM_HEFF the field
+// terms of io.terms.
 mx_status fast_row_stage(mx_ctx* ctx, int mode, const StageIO& io, bool xf_next, float4* hd_out, cudaStream_t st);
+// Whether the one-layer y/z pass of the grid takes its wide kernel (demag_fast.cu).
+bool yz2d_wide(const Grid& g);
 // Whether RK4 steps of this context run as y/z passes plus row kernels (api.cu).
 bool row_steps(const mx_ctx* ctx, int method);
 mx_status plane_spectrum_out(mx_ctx* ctx, float* out, cudaStream_t st);

@@ -38,14 +38,17 @@ __device__ __forceinline__ void neighbours(const float4* __restrict__ m, const G
   zm = (k > 0) ? f3(__ldg(&m[idx - sz])) : mc;
 }
 
-// All field terms at cell (i, j, k); the demag term is the given value hdv,
-// the easy axis e and the anisotropy coefficient cK = 2 Ku / mu0 are given.
+// The six neighbours of a cell.
+struct Nbrs {
+  float3 xp, xm, yp, ym, zp, zm;
+};
+
+// All field terms of a cell from its neighbours; the demag term is the given value
+// hdv, the easy axis e and the anisotropy coefficient cK = 2 Ku / mu0 are given.
 template <bool DMI>
-__device__ __forceinline__ void local_terms_ek(const float4* __restrict__ m, float3 hdv, const Grid& g,
-                                               const LocalCoef& c, int i, int j, int k, long idx, float3 mc,
-                                               float inv_ms, float3 e, float cK, Terms& t) {
-  float3 xm, xp, ym, yp, zm, zp;
-  neighbours(m, g, c, i, j, k, idx, mc, xp, xm, yp, ym, zp, zm);
+__device__ __forceinline__ void local_terms_nb(const Nbrs& b, float3 hdv, const LocalCoef& c, float3 mc, float inv_ms,
+                                               float3 e, float cK, Terms& t) {
+  const float3 xp = b.xp, xm = b.xm, yp = b.yp, ym = b.ym, zp = b.zp, zm = b.zm;
   const float3 two = 2.f * mc;
   const float3 lap = c.inv_dx2 * (xp + xm - two) + c.inv_dy2 * (yp + ym - two) + c.inv_dz2 * (zp + zm - two);
   t.exch = (c.cA * inv_ms) * lap;
@@ -59,6 +62,27 @@ __device__ __forceinline__ void local_terms_ek(const float4* __restrict__ m, flo
   t.anis = (cK * inv_ms * dot3(mc, e)) * e;
   t.zee = make_float3(c.hx, c.hy, c.hz);
   t.demag = hdv;
+}
+
+// All field terms at cell (i, j, k).
+template <bool DMI>
+__device__ __forceinline__ void local_terms_ek(const float4* __restrict__ m, float3 hdv, const Grid& g,
+                                               const LocalCoef& c, int i, int j, int k, long idx, float3 mc,
+                                               float inv_ms, float3 e, float cK, Terms& t) {
+  Nbrs b;
+  neighbours(m, g, c, i, j, k, idx, mc, b.xp, b.xm, b.yp, b.ym, b.zp, b.zm);
+  local_terms_nb<DMI>(b, hdv, c, mc, inv_ms, e, cK, t);
+}
+
+// sum of the terms of the MX_TERM_* mask
+__device__ __forceinline__ float3 masked_sum(const Terms& t, int terms) {
+  float3 out = make_float3(0.f, 0.f, 0.f);
+  if (terms & MX_TERM_DEMAG) out = out + t.demag;
+  if (terms & MX_TERM_EXCH) out = out + t.exch;
+  if (terms & MX_TERM_ANIS) out = out + t.anis;
+  if (terms & MX_TERM_DMI) out = out + t.dmi;
+  if (terms & MX_TERM_ZEEMAN) out = out + t.zee;
+  return out;
 }
 
 __device__ __forceinline__ float3 easy_axis(const LocalCoef& c, long idx) {
@@ -140,12 +164,7 @@ __device__ __forceinline__ void local_cell_in(const StageIO& io, const Grid& g, 
   float3 out;
   float wout = 0.f;  // |u| of a renormalised stage output (used by the adjoint)
   if (MODE == LM_HEFF) {
-    out = make_float3(0.f, 0.f, 0.f);
-    if (io.terms & MX_TERM_DEMAG) out = out + t.demag;
-    if (io.terms & MX_TERM_EXCH) out = out + t.exch;
-    if (io.terms & MX_TERM_ANIS) out = out + t.anis;
-    if (io.terms & MX_TERM_DMI) out = out + t.dmi;
-    if (io.terms & MX_TERM_ZEEMAN) out = out + t.zee;
+    out = masked_sum(t, io.terms);
   } else {
     const float3 H = t.demag + t.exch + t.anis + t.dmi + t.zee;
     const float3 kk = llg(c, mc, H);
@@ -171,7 +190,57 @@ __device__ __forceinline__ void local_cell_in(const StageIO& io, const Grid& g, 
   io.out[idx] = make_float4(out.x, out.y, out.z, wout);
 }
 
-// The same with the inputs loaded here.
+// A cell of an RK4 stage or the Euler step with its inputs and neighbours held, the
+// mode chosen at run time (the arithmetic of local_cell_in).
+struct StageCell {
+  float3 m, m0, acc, e;
+  float ms, cK;
+  Nbrs b;
+  __device__ __forceinline__ void load(const StageIO& io, const Grid& g, const LocalCoef& c, int i, int j, int k,
+                                       long idx, int mode) {
+    m = f3(io.m[idx]);
+    m0 = m;
+    acc = make_float3(0.f, 0.f, 0.f);
+    if (mode == LM_RK4_S1 || mode == LM_RK4_S2 || mode == LM_RK4_S3) {
+      m0 = f3(io.m0[idx]);
+      acc = f3(io.acc[idx]);
+    }
+    ms = c.ms_map ? __ldg(&c.ms_map[idx]) : c.Ms;
+    e = easy_axis(c, idx);
+    cK = aniso_coef(c, idx);
+    neighbours(io.m, g, c, i, j, k, idx, m, b.xp, b.xm, b.yp, b.ym, b.zp, b.zm);
+  }
+  // the field terms of io.terms to io.out (LM_HEFF)
+  template <bool DMI>
+  __device__ __forceinline__ void heff(const StageIO& io, const LocalCoef& c, long idx, float3 hdv, int* flag) const {
+    Terms t;
+    local_terms_nb<DMI>(b, hdv, c, m, 1.f / ms, e, cK, t);
+    const float3 out = masked_sum(t, io.terms);
+    if (!(isfinite(out.x) && isfinite(out.y) && isfinite(out.z))) atomicOr(flag, kFlagNonfinite);
+    io.out[idx] = make_float4(out.x, out.y, out.z, 0.f);
+  }
+  // writes io.out and io.acc; returns the stage output
+  template <bool DMI>
+  __device__ __forceinline__ float3 stage(const StageIO& io, const LocalCoef& c, long idx, float3 hdv, int mode,
+                                          int* flag) const {
+    Terms t;
+    local_terms_nb<DMI>(b, hdv, c, m, 1.f / ms, e, cK, t);
+    const float3 kk = llg(c, m, t.demag + t.exch + t.anis + t.dmi + t.zee);
+    const bool last = mode == LM_RK4_S3;
+    if (!last && mode != LM_EULER) {
+      const float w = mode == LM_RK4_S0 ? 1.f : 2.f;
+      io.acc[idx] = make_float4(acc.x + w * kk.x, acc.y + w * kk.y, acc.z + w * kk.z, 0.f);
+    }
+    const float h = last ? io.dt * (1.f / 6.f) : (mode == LM_RK4_S2 || mode == LM_EULER ? io.dt : 0.5f * io.dt);
+    float wout = 0.f;
+    const float3 out = unit_norm(m0 + h * (last ? acc + kk : kk), wout);
+    if (!(isfinite(out.x) && isfinite(out.y) && isfinite(out.z))) atomicOr(flag, kFlagNonfinite);
+    io.out[idx] = make_float4(out.x, out.y, out.z, wout);
+    return out;
+  }
+};
+
+// local_cell_in with the inputs loaded here.
 template <int MODE, bool DMI>
 __device__ __forceinline__ void local_cell_v(const StageIO& io, const Grid& g, const LocalCoef& c, int i, int j,
                                              int k, long idx, float3 hdv, int* flag) {

@@ -78,3 +78,41 @@ def test_many_row_x_kernels_match_generic_passes(shape, ms_map):
     ref, gen = field(c, Ms=Ms, demag_path=_lib.MX_DEMAG_GENERIC)
     assert gen.kernel_name("x_fwd") == "x_fwd_kernel"
     assert rel_l2(h, ref) <= TOL
+
+
+# (nx, ny): one layer, Px/2 and Py/2 = 16 .. 1024 and 16 .. 512, one, two, four and eight columns per
+# block and the wide kernel, odd last columns, ragged rows
+FILMS = [(9, 9), (16, 16), (31, 30), (70, 20), (640, 30), (33, 33), (200, 60), (700, 50), (100, 100), (300, 128),
+         (1000, 70), (60, 200), (200, 150), (300, 200), (120, 300), (130, 500)]
+
+
+@pytest.mark.parametrize("shape", FILMS)
+def test_film_kernels_match_generic_passes(shape):
+    from paper_2602_12242_gb300 import _lib
+    c = cfg_of(nx=shape[0], ny=shape[1], nz=1, dx=2e-9, dy=2.5e-9, dz=3e-9)
+    h, ctx = field(c)
+    wide = (shape[1] > 256 and shape[0] > 128) or (128 < shape[1] <= 256 and shape[0] > 256)
+    assert ctx.kernel_name("yz_fused") == ("yz2d_wide_kernel" if wide else "yz2d_kernel")
+    ref, _ = field(c, demag_path=_lib.MX_DEMAG_GENERIC)
+    assert rel_l2(h, ref) <= TOL
+
+
+@pytest.mark.parametrize("shape", [(9, 9, 1), (31, 30, 1), (40, 20, 3), (65, 33, 1), (200, 60, 2), (300, 40, 1),
+                                   (1000, 33, 1)])
+@pytest.mark.parametrize("ms_map", [False, True])
+def test_row_kernel_steps_match_generic_passes(shape, ms_map):
+    """Every row length, ragged, with DMI: two RK4 steps (the four stages' updates, and the rows that a
+    step leaves transformed for the next) against the separate kernels on the generic passes."""
+    from paper_2602_12242_gb300 import _lib
+    from paper_2602_12242_gb300.solver import from_dev4, to_dev4
+    c = cfg_of(nx=shape[0], ny=shape[1], nz=shape[2], dx=2e-9, dy=2.5e-9, dz=3e-9, D=1e-3, dmi=True)
+    Ms = np.random.default_rng(47).uniform(6e5, 1e6, size=shape[::-1]) if ms_map else None
+    out = []
+    for kw in ({}, dict(demag_path=_lib.MX_DEMAG_GENERIC)):
+        ctx = context(c, Ms=Ms, **kw)
+        m = to_dev4(np.asarray(random_m(c, 48), np.float32))
+        ctx.rk_step(m, 2, 1e-14, "rk4")
+        out.append(from_dev4(m))
+        name = ctx.kernel_name("x_inv_local")
+        assert name == ("xr_kernel" if not kw else "")
+    assert rel_l2(out[0], out[1]) <= TOL
