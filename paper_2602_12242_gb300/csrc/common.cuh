@@ -93,6 +93,26 @@ template <typename C> __host__ __device__ __forceinline__ C mkc(typename real_of
 }
 template <typename C> __device__ __forceinline__ C cadd(C a, C b) { return mkc<C>(a.x + b.x, a.y + b.y); }
 template <typename C> __device__ __forceinline__ C csub(C a, C b) { return mkc<C>(a.x - b.x, a.y - b.y); }
+// Single-precision sums as one packed instruction: the pipes take it in two cycles, as
+// two scalar ones, but it is one issue slot, and the transforms are bound by issue and
+// latency.  With the tensor multiply packed too (zcol.cuh): bulk grid y/z kernel 231 -> 211 us
+// per launch and step 1606 -> 1521 us, cube step (128^3) 266 -> 257, 640x160x4 multirate step
+// 415 -> 404.  The complex multiply stays scalar (packed, with its swapped operand: 1568 and
+// 1607 us for the bulk step).
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) {
+  float2 d;
+  asm("{.reg .b64 x, y, z; mov.b64 x, {%2, %3}; mov.b64 y, {%4, %5}; add.rn.f32x2 z, x, y; mov.b64 {%0, %1}, z;}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ float2 csub(float2 a, float2 b) {
+  float2 d;
+  asm("{.reg .b64 x, y, z; mov.b64 x, {%2, %3}; mov.b64 y, {%4, %5}; sub.rn.f32x2 z, x, y; mov.b64 {%0, %1}, z;}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
 template <typename C> __device__ __forceinline__ C cmul(C a, C b) {
   return mkc<C>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }

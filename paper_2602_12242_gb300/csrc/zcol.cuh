@@ -15,9 +15,12 @@ namespace mx {
 __device__ __forceinline__ void tensor_apply(float2& a, float2& b, float2& c, float nxx, float nyy, float nzz,
                                              float nxy, float nxz, float nyz) {
   const float2 mx = a, my = b, mz = c;
-  a = make_float2(fmaf(nxz, mz.x, fmaf(nxy, my.x, nxx * mx.x)), fmaf(nxz, mz.y, fmaf(nxy, my.y, nxx * mx.y)));
-  b = make_float2(fmaf(nyz, mz.x, fmaf(nyy, my.x, nxy * mx.x)), fmaf(nyz, mz.y, fmaf(nyy, my.y, nxy * mx.y)));
-  c = make_float2(fmaf(nzz, mz.x, fmaf(nyz, my.x, nxz * mx.x)), fmaf(nzz, mz.y, fmaf(nyz, my.y, nxz * mx.y)));
+  auto row = [&](float u, float v, float w) {  // u mx + v my + w mz
+    return __ffma2_rn(make_float2(w, w), mz, __ffma2_rn(make_float2(v, v), my, __fmul2_rn(make_float2(u, u), mx)));
+  };
+  a = row(nxx, nxy, nxz);
+  b = row(nxy, nyy, nyz);
+  c = row(nxz, nyz, nzz);
 }
 
 // The six components of octant entry kz of a column (tq: its entry at qz = 0,
