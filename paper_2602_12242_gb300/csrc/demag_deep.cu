@@ -387,7 +387,11 @@ template <int L> static mx_status deep_z_run(mx_ctx* ctx, cudaStream_t st, bool 
   // exchange once more (zc at 256x256x32: 88 us against 88, at 64^3 20 against
   // 21; at 128^3 133 against 119, at 30x200x200 186 against 152).
   constexpr bool SPLIT = L > 64;
-  auto k = SPLIT ? deep_z3_kernel<L> : deep_z_kernel<L>;
+  void (*k)(float2*, Grid, const float*, const float2*);
+  if constexpr (SPLIT)
+    k = deep_z3_kernel<L>;
+  else
+    k = deep_z_kernel<L>;
   const size_t sm = D::smem(6 * D::T);
   if (setup) {
     MX_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
