@@ -93,7 +93,8 @@ static mx_status check_ctx(const mx_ctx* ctx) {
 static void invalidate_graph(mx_ctx* ctx) {
   adjoint_invalidate_graphs(ctx);
   if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
-  ctx->graph = nullptr;
+  if (ctx->pair) cudaGraphExecDestroy(ctx->pair);
+  ctx->graph = ctx->pair = nullptr;
   ctx->graph_m = nullptr;
   ctx->graph_method = -1;
 }
@@ -120,6 +121,23 @@ static mx_status lead_x_pass(mx_ctx* ctx, const float4* m, cudaStream_t st) {
   return fast_x_pass(ctx, m, nullptr, false, st);
 }
 
+// One Euler step from `from` to `to` on stream st (lead, tail: as enqueue_step).
+static mx_status enqueue_euler(mx_ctx* ctx, const float4* from, float4* to, double dt, cudaStream_t st, bool lead,
+                               bool tail) {
+  const bool demag = ctx->p.demag != 0;
+  float4* hd = demag ? ctx->hd : nullptr;
+  StageIO io{from, hd, from, ctx->acc, to, (float)dt, MX_TERM_ALL};
+  if (row_steps(ctx, MX_EULER)) {
+    if (lead) MX_TRY(lead_x_pass(ctx, from, st));
+    MX_TRY(demag_yz(ctx, st));
+    ProfScope ps(ctx, KID_X_INV_LOCAL, st);
+    return fast_row_stage(ctx, LM_EULER, io, tail, nullptr, st);
+  }
+  if (demag && ctx->xlocal) return plane_stage_xlocal(ctx, LM_EULER, io, st);
+  if (demag) MX_TRY(demag_field(ctx, from, hd, st));
+  return local_stage(ctx, LM_EULER, io, st);
+}
+
 // One time step on stream st.  m is the caller's field (step start, updated
 // in place).  With row kernels (row_steps), `lead` runs the forward x pass of
 // m first (else w1 must already hold it) and `tail` has the last stage leave
@@ -131,18 +149,7 @@ static mx_status enqueue_step(mx_ctx* ctx, float4* m, double dt, int method, cud
   float4* hd = demag ? ctx->hd : nullptr;
   const bool xlocal = demag && ctx->xlocal;
   if (method == MX_EULER) {
-    StageIO io{m, hd, m, ctx->acc, ctx->sa, (float)dt, MX_TERM_ALL};
-    if (row_steps(ctx, method)) {
-      if (lead) MX_TRY(lead_x_pass(ctx, m, st));
-      MX_TRY(demag_yz(ctx, st));
-      ProfScope ps(ctx, KID_X_INV_LOCAL, st);
-      MX_TRY(fast_row_stage(ctx, LM_EULER, io, tail, nullptr, st));
-    } else if (xlocal) {
-      MX_TRY(plane_stage_xlocal(ctx, LM_EULER, io, st));
-    } else {
-      if (demag) MX_TRY(demag_field(ctx, m, hd, st));
-      MX_TRY(local_stage(ctx, LM_EULER, io, st));
-    }
+    MX_TRY(enqueue_euler(ctx, m, ctx->sa, dt, st, lead, tail));
     return copy_field(ctx, m, ctx->sa, st);
   }
   // RK4: m -> sa -> sb -> sa -> m
@@ -504,40 +511,55 @@ static mx_status check_step_args(mx_ctx* ctx, const float* m, int nsteps, double
   return MX_OK;
 }
 
+// The graph of one step, or with `two` of two Euler steps.  With row kernels it starts
+// from w1 and leaves it for the next.
+static mx_status capture_steps(mx_ctx* ctx, float4* m, double dt, int method, bool two, cudaGraphExec_t* exec) {
+  cudaGraph_t graph = nullptr;
+  MX_CUDA_TRY(cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
+  mx_status s;
+  if (two) {
+    s = enqueue_euler(ctx, m, ctx->sa, dt, ctx->cap_stream, false, true);
+    if (s == MX_OK) s = enqueue_euler(ctx, ctx->sa, m, dt, ctx->cap_stream, false, true);
+  } else {
+    s = enqueue_step(ctx, m, dt, method, ctx->cap_stream, false, true);
+  }
+  cudaError_t e = cudaStreamEndCapture(ctx->cap_stream, &graph);
+  if (s != MX_OK) {
+    if (graph) cudaGraphDestroy(graph);
+    return s;
+  }
+  if (e != cudaSuccess) {
+    set_error(std::string("mx_rk_step: capture failed: ") + cudaGetErrorString(e));
+    return MX_ERR_CUDA;
+  }
+  e = cudaGraphInstantiate(exec, graph, 0);
+  cudaGraphDestroy(graph);
+  if (e != cudaSuccess) {
+    *exec = nullptr;
+    set_error(std::string("mx_rk_step: instantiate failed: ") + cudaGetErrorString(e));
+    return MX_ERR_CUDA;
+  }
+  return MX_OK;
+}
+
 mx_status mx_rk_step(mx_ctx* ctx, float* m, int nsteps, double dt, int method, mx_stream_t stream) {
   MX_TRY(check_step_args(ctx, m, nsteps, dt, method));
   cudaStream_t st = (cudaStream_t)stream;
   if (nsteps == 0) return MX_OK;
   if (method == MX_MRI) MX_TRY(mri_reserve(ctx));
   MX_TRY(normalize_field(ctx, (float4*)m, st));
-  if (!ctx->graph || ctx->graph_m != m || ctx->graph_dt != dt || ctx->graph_method != method) {
-    invalidate_graph(ctx);
-    cudaGraph_t graph = nullptr;
-    MX_CUDA_TRY(cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
-    // with row kernels the graph step starts from w1 and leaves it for the next
-    mx_status s = enqueue_step(ctx, (float4*)m, dt, method, ctx->cap_stream, false, true);
-    cudaError_t e = cudaStreamEndCapture(ctx->cap_stream, &graph);
-    if (s != MX_OK) {
-      if (graph) cudaGraphDestroy(graph);
-      return s;
-    }
-    if (e != cudaSuccess) {
-      set_error(std::string("mx_rk_step: capture failed: ") + cudaGetErrorString(e));
-      return MX_ERR_CUDA;
-    }
-    e = cudaGraphInstantiate(&ctx->graph, graph, 0);
-    cudaGraphDestroy(graph);
-    if (e != cudaSuccess) {
-      ctx->graph = nullptr;
-      set_error(std::string("mx_rk_step: instantiate failed: ") + cudaGetErrorString(e));
-      return MX_ERR_CUDA;
-    }
-    ctx->graph_m = m;
-    ctx->graph_dt = dt;
-    ctx->graph_method = method;
-  }
+  if (ctx->graph_m != m || ctx->graph_dt != dt || ctx->graph_method != method) invalidate_graph(ctx);
+  ctx->graph_m = m;
+  ctx->graph_dt = dt;
+  ctx->graph_method = method;
+  // Two Euler steps go to sa and back, without the copy that ends a single one (128^3: 11
+  // us of 262 a step).
+  const int pairs = method == MX_EULER ? nsteps / 2 : 0;
+  if (pairs > 0 && !ctx->pair) MX_TRY(capture_steps(ctx, (float4*)m, dt, method, true, &ctx->pair));
+  if (nsteps > 2 * pairs && !ctx->graph) MX_TRY(capture_steps(ctx, (float4*)m, dt, method, false, &ctx->graph));
   if (row_steps(ctx, method)) MX_TRY(lead_x_pass(ctx, (const float4*)m, st));
-  for (int s = 0; s < nsteps; ++s) MX_CUDA_TRY(cudaGraphLaunch(ctx->graph, st));
+  for (int s = 0; s < pairs; ++s) MX_CUDA_TRY(cudaGraphLaunch(ctx->pair, st));
+  for (int s = 2 * pairs; s < nsteps; ++s) MX_CUDA_TRY(cudaGraphLaunch(ctx->graph, st));
   return MX_OK;
 }
 

@@ -233,8 +233,8 @@ struct mx_ctx {
   int* flag = nullptr;            // non-finite flag
   double* ered = nullptr;         // energy accumulators (5)
 
-  // CUDA graph cache for mx_rk_step
-  cudaGraphExec_t graph = nullptr;
+  // CUDA graph cache for mx_rk_step: a step, and two Euler steps
+  cudaGraphExec_t graph = nullptr, pair = nullptr;
   const float* graph_m = nullptr;
   double graph_dt = 0.0;
   int graph_method = -1;

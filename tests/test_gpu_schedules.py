@@ -116,3 +116,22 @@ def test_row_kernel_steps_match_generic_passes(shape, ms_map):
         name = ctx.kernel_name("x_inv_local")
         assert name == ("xr_kernel" if not kw else "")
     assert rel_l2(out[0], out[1]) <= TOL
+
+
+@pytest.mark.parametrize("shape", [(40, 20, 1), (33, 16, 3), (40, 33, 64), (64, 64, 16)])
+@pytest.mark.parametrize("n", [2, 3, 4])
+def test_euler_step_pairs_equal_single_steps(shape, n):
+    """Row-kernel, deep and plane grids: a call of n steps (pairs of steps and the odd one) against n
+    calls of one step, also when the two kinds of call alternate.  A call renormalises m first, which
+    changes a component by a few FP32 roundings (6e-8) per call."""
+    from paper_2602_12242_gb300.solver import from_dev4, to_dev4
+    c = cfg_of(nx=shape[0], ny=shape[1], nz=shape[2], dx=2e-9, dy=2.5e-9, dz=3e-9)
+    ctx = context(c)
+    m0 = np.asarray(random_m(c, 49), np.float32)
+    a, b = to_dev4(m0), to_dev4(m0)
+    for _ in range(2):
+        ctx.rk_step(a, n, 1e-14, "euler")
+        ctx.rk_step(a, 1, 1e-14, "euler")
+    for _ in range(2 * (n + 1)):
+        ctx.rk_step(b, 1, 1e-14, "euler")
+    assert np.abs(from_dev4(a) - from_dev4(b)).max() <= 2e-6
