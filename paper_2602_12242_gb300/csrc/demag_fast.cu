@@ -385,10 +385,10 @@ __global__ void __launch_bounds__(Yz2d<LH, T, PAIR>::NT, Yz2d<LH, T, PAIR>::MB)
     }
   }
   __syncthreads();
-  for (int e = tid; e < 3 * T * ny; e += NT) {
-    const int t = e % T, y = (e / T) % ny, c = e / (T * ny);
+  for (int e = tid; e < 3 * T * LH; e += NT) {
+    const int t = e % T, y = (e / T) % LH, c = e / (T * LH);
     const int kx = kx0 + t;
-    if (kx >= g.Hx) continue;
+    if (y >= ny || kx >= g.Hx) continue;
     const float2* H = sm + NO * D::half + (c * T + t) * 2 * PITCH + L::at(y);
     w1[c * wc + (long)y * g.Hx + kx] = PAIR ? H[0] : cadd(H[0], H[PITCH]);
   }
@@ -494,10 +494,10 @@ __global__ void __launch_bounds__(NT) yz2d_wide_kernel(float2* __restrict__ w1, 
   __syncthreads();
   if (tid < NF) line_fft<E, S, true, true, true>(sm + (tid / S) * PITCH, tid % S, twS);
   __syncthreads();
-  for (int e = tid; e < 3 * T * ny; e += NT) {
-    const int t = e % T, y = (e / T) % ny, c = e / (T * ny);
+  for (int e = tid; e < 3 * T * LH; e += NT) {
+    const int t = e % T, y = (e / T) % LH, c = e / (T * LH);
     const int kx = kx0 + t;
-    if (kx >= g.Hx) continue;
+    if (y >= ny || kx >= g.Hx) continue;
     const float2* L = sm + ((c * T + t) * 2) * PITCH;
     w1[c * wc + (long)y * g.Hx + kx] = cadd(L[y], cmul(L[PITCH + y], cconj(twS2[y])));
   }

@@ -17,11 +17,12 @@
 // three 8-byte loads and neighbouring columns are contiguous.
 //
 // Bound: the latency of that chain (load, two line FFTs, column, store) at two
-// to four blocks per SM.  Measured (one evaluation, kernel alone): 32x32x4
-// 14.1 -> 3.9 us and 201x77x3 73.4 -> 9 us against yz_fused_kernel; 640x160x4
-// 107 -> 52 us, 256x256x4 32 -> 19 us and 256x256x8 42 -> 35 us against the
-// four-CTA plane kernel, whose cluster barriers and small shares of a plane
-// cost more than they save where a plane fits one block.
+// to four blocks per SM, and on large grids instruction issue (60 % at 640x160x4).
+// Measured (one evaluation, kernel alone): 32x32x4 14.1 -> 3.9 us and 201x77x3 73.4
+// -> 9 us against yz_fused_kernel; 640x160x4 107 -> 42 us (49 with divisions by
+// run-time sizes in the load and store loops), 256x256x4 32 -> 16 us and 256x256x8
+// 42 -> 35 us against the four-CTA plane kernel, whose cluster barriers and small
+// shares of a plane cost more than they save where a plane fits one block.
 #include <math.h>
 
 #include "common.cuh"
@@ -33,7 +34,7 @@
 namespace mx {
 
 // (64 registers per thread, so two 512-thread blocks share an SM, where that spills
-// at most a few words: 640x160x4 62 -> 52 us)
+// at most a few words: 640x160x4 62 -> 52 us when measured)
 template <int E, int S, int P, int T, int NT, bool KM>
 __global__ void __launch_bounds__(NT, NT == 512 && E <= 16 && P <= 8 ? 2 : 1) yz3_kernel(const float2* win, float2* wout, Grid g, const float* __restrict__ nhk,
                                                  const float2* __restrict__ twH, const float2* __restrict__ twPy) {
@@ -51,13 +52,15 @@ __global__ void __launch_bounds__(NT, NT == 512 && E <= 16 && P <= 8 ? 2 : 1) yz
   float2* dummy = twS2 + LH;            // scratch line for idle thread groups
   const int kx0 = blockIdx.x * T;
   const int tid = threadIdx.x;
-  // element (cz, y) of kx column t, element e of the block's load and store loops
+  // element (cz, y) of kx column t, element e of the block's load and store loops (LH, not
+  // ny, values per line and KM with one column: no division by a run-time value)
+  static_assert(!KM || T == 1, "kx-major blocks hold one column");
   auto wi = [&](int t, int y, int cz) {
-    return KM ? ((long)(kx0 + t) * 3 * nz + cz) * ny + y : ((long)cz * ny + y) * Hx + kx0 + t;
+    return KM ? ((long)kx0 * 3 * nz + cz) * ny + y : ((long)cz * ny + y) * Hx + kx0 + t;
   };
-  auto et = [&](int e) { return KM ? e / (3 * nz * LH) : e % T; };
-  auto ey = [&](int e) { return KM ? e % LH : (e / T) % LH; };
-  auto ecz = [&](int e) { return KM ? (e / LH) % (3 * nz) : e / (T * LH); };
+  auto et = [&](int e) { return e % T; };
+  auto ey = [&](int e) { return (e / T) % LH; };
+  auto ecz = [&](int e) { return e / (T * LH); };
   for (int q = tid; q < LH; q += NT) {
     twS[q] = __ldg(&twH[(q % S) * (q / S)]);
     twS2[q] = __ldg(&twPy[q]);

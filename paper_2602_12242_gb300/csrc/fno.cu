@@ -134,21 +134,38 @@ __device__ __forceinline__ void fno_row_dft(const float* vs, int P, int Wp, int 
   }
 }
 
+// Element q = threadIdx.x, + blockDim.x, ... of rows of n: its row and place, without a
+// division per element.
+struct RowWalk {
+  int r, c, dr, dc, n;
+  __device__ __forceinline__ explicit RowWalk(int n) : n(n) {
+    r = threadIdx.x / n;
+    c = threadIdx.x - r * n;
+    dr = blockDim.x / n;
+    dc = blockDim.x - dr * n;
+  }
+  __device__ __forceinline__ void next() {
+    r += dr;
+    c += dc;
+    if (c >= n) {
+      c -= n;
+      ++r;
+    }
+  }
+};
+
 // The twiddle rows into shared memory (pitch P): constants, so before the
 // dependency wait, which hides their latency where a launch has few blocks.
 __device__ __forceinline__ void fno_stage_tw(float* dst, const float* __restrict__ tw, int Wp, int P, int K) {
-  const int n4 = Wp / 4;
-  for (int q = threadIdx.x; q < 2 * K * n4; q += blockDim.x)
-    *reinterpret_cast<float4*>(dst + q / n4 * P + q % n4 * 4) = ldg4(tw + (long)(q / n4) * Wp + q % n4 * 4);
+  for (RowWalk q(Wp / 4); q.r < 2 * K; q.next())
+    *reinterpret_cast<float4*>(dst + q.r * P + q.c * 4) = ldg4(tw + q.r * Wp + q.c * 4);
 }
 
 // 16-byte asynchronous copies of a row's planes into shared memory, one group
 __device__ __forceinline__ void fno_copy_row(float* vs, const float* v, int Wp, int P) {
-  const int n4 = Wp / 4;
-  for (int q = threadIdx.x; q < kFC * n4; q += blockDim.x) {
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(vs + q / n4 * P + q % n4 * 4);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(v + (long)(q / n4) * Wp + q % n4 * 4)
-                 : "memory");
+  for (RowWalk q(Wp / 4); q.r < kFC; q.next()) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(vs + q.r * P + q.c * 4);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(v + q.r * Wp + q.c * 4) : "memory");
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
