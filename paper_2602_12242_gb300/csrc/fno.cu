@@ -683,7 +683,7 @@ __device__ __forceinline__ void fno_proj_weights(float* Q1t, float* q1s, float* 
 __device__ __forceinline__ void fno_load_tile(float* vs, const float* __restrict__ v, long tile, long groups, int Wp) {
   const int n4 = Wp / 4, g = threadIdx.x % (kPT / 4);
   const long gg = tile * (kPT / 4) + g;
-  const long r = gg / n4;
+  const long r = (int)gg / n4;  // (a group has 6 kB of activations, so their number fits 31 bits)
   const float* src = v + r * kFC * Wp + (gg - r * n4) * 4;
 #pragma unroll
   for (int q = 0; q < kFC * (kPT / 4) / kPN; ++q) {
@@ -695,7 +695,7 @@ __device__ __forceinline__ void fno_load_tile(float* vs, const float* __restrict
 // cell i of the tile: its index in the compact [row][W] fields, -1 for padding
 __device__ __forceinline__ long fno_cell(long tile, int i, long groups, int W, int Wp) {
   const long gg = tile * (kPT / 4) + i / 4;
-  const long r = gg / (Wp / 4);
+  const long r = (int)gg / (Wp / 4);
   const int x = (int)(gg - r * (Wp / 4)) * 4 + i % 4;
   return gg < groups && x < W ? r * W + x : -1;
 }
@@ -903,7 +903,7 @@ __global__ void __launch_bounds__(kPN, 2)
       }
       reduce_scatter<64, 3, 0>(a, lane);  // entries q = 8 k + sp: channel k, cell entry sp
       const long gg = tile * (kPT / 4) + (sp < 4 ? 0 : 8) + xq;
-      const long r = gg / (Wp / 4);
+      const long r = (int)gg / (Wp / 4);
       if (gg < groups) {
         float* dst = dv + (r * kFC + 8 * ig) * Wp + (gg - r * (Wp / 4)) * 4 + (sp & 3);
         // (dz is zero in the padding, so dv is too)
