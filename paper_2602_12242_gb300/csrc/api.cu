@@ -362,7 +362,8 @@ mx_status mx_destroy(mx_ctx* ctx) {
 
 mx_status mx_inject_wait_timeout(mx_ctx* ctx, int on) {
   MX_TRY(check_ctx(ctx));
-  if (on && !(ctx->plane && !ctx->quad && (ctx->g.ny & 1) == 0 && !ctx->surrogate && !ctx->fno)) {
+  // (the plane path's y/z kernel is the two-CTA one unless yz3 or quad is set)
+  if (on && !(ctx->plane && !ctx->yz3 && !ctx->quad && (ctx->g.ny & 1) == 0 && !ctx->surrogate && !ctx->fno)) {
     set_error("mx_inject_wait_timeout: needs the two-CTA plane kernel with bulk copies (MX_DEMAG_PLANE_PAIR, even ny)");
     return MX_ERR_UNSUPPORTED;
   }

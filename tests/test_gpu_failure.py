@@ -52,3 +52,14 @@ def test_wait_timeout_hook_needs_the_two_cta_kernel():
     with pytest.raises(MxError) as ei:
         _lib.mx_inject_wait_timeout(ctx.h, 1)
     assert ei.value.status == _lib.MX_ERR_UNSUPPORTED
+
+
+def test_wait_timeout_hook_refuses_the_few_layer_kernel():
+    """A kx-major grid whose y/z pass is the few-layer kernel (no bulk-copy barrier)."""
+    from paper_2602_12242_gb300 import MxError, _lib
+    c = cfg_of(nx=70, ny=128, nz=5)
+    ctx = context(c)
+    assert (ctx.kernel_name("x_fwd"), ctx.kernel_name("yz_fused")) == ("xfk_kernel", "yz3_kernel")
+    with pytest.raises(MxError) as ei:
+        _lib.mx_inject_wait_timeout(ctx.h, 1)
+    assert ei.value.status == _lib.MX_ERR_UNSUPPORTED
