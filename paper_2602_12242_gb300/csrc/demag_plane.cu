@@ -653,6 +653,15 @@ static mx_status plane_yz(mx_ctx* ctx, cudaStream_t st) {
   return ctx->quad ? quad_pass(ctx, st, false) : yzh_pass(ctx, st, false);
 }
 
+// Plane grids that the four-CTA y/z kernel serves better than the few-layer one: with at
+// most one kx column to two SMs a block per column leaves the rest of the chip idle, which
+// costs more than the cluster's barriers where a column's z and y stages are long.  RK4
+// step at 65 columns, few-layer and four-CTA: 33x128x8 (Py/2 = 128, Pz = 16) 68.8 and 62.1
+// us, 33x109x7 66.8 and 61.3, 33x256x8 (256, 16) 88.5 and 83.2, 33x280x3 (512, 8) 76.9 and
+// 73.3; the other way 33x256x4 (256, 8) 62.7 and 66.8, 33x500x2 (512, 4) 64.7 and 67.8, and
+// at 129 columns all of them, 80x128x8 93.4 and 98.1 the closest.
+static bool quad_first(const Grid& g) { return 2 * g.Hx <= kSMs && (g.Pz >= 16 || (long)g.Py * g.Pz >= 8192); }
+
 mx_status plane_setup(mx_ctx* ctx) {
   MX_TRY(upload_w32());
   const int path = ctx->p.demag_path;
@@ -661,10 +670,12 @@ mx_status plane_setup(mx_ctx* ctx) {
   // the four-CTA y/z kernel where it fits, else the two-CTA one
   // (MX_DEMAG_PLANE_PAIR forces the two-CTA kernel)
   // the few-layer y/z kernel wherever it fits, in place on the small-grid
-  // layout unless the grid's x passes are the kx-major ones
-  ctx->yz3 = path == MX_DEMAG_AUTO && ctx->fast_x && yz3_pass(ctx, xk, nullptr, true) == MX_OK;
+  // layout unless the grid's x passes are the kx-major ones (and quad_first)
+  auto quad = [&] { return xk && path != MX_DEMAG_PLANE_PAIR && quad_pass(ctx, nullptr, true) == MX_OK; };
+  ctx->yz3 = path == MX_DEMAG_AUTO && ctx->fast_x && !(quad_first(ctx->g) && quad()) &&
+             yz3_pass(ctx, xk, nullptr, true) == MX_OK;
   if (ctx->yz3 && !xk) ctx->fused_yz = true;
-  ctx->quad = xk && !ctx->yz3 && path != MX_DEMAG_PLANE_PAIR && quad_pass(ctx, nullptr, true) == MX_OK;
+  ctx->quad = !ctx->yz3 && quad();
   ctx->plane = ctx->quad || (xk && ctx->yz3) || (xk && yzh_pass(ctx, nullptr, true) == MX_OK);
   ctx->deep = path == MX_DEMAG_AUTO && ctx->fast_x && !ctx->plane && !ctx->fused_yz && deep_setup(ctx);
   ctx->g.oct4 = ctx->quad ? 1 : (ctx->deep ? 2 : 0);

@@ -135,3 +135,17 @@ def test_euler_step_pairs_equal_single_steps(shape, n):
     for _ in range(2 * (n + 1)):
         ctx.rk_step(b, 1, 1e-14, "euler")
     assert np.abs(from_dev4(a) - from_dev4(b)).max() <= 2e-6
+
+
+# (nx, ny, nz, kernel): 65 kx columns on the plane path, both sides of the line between the four-CTA and
+# the few-layer kernel, and 129 columns
+@pytest.mark.parametrize("nx,ny,nz,kernel", [
+    (33, 128, 8, "yzq_kernel"), (64, 65, 5, "yzq_kernel"), (50, 200, 5, "yzq_kernel"), (40, 300, 3, "yzq_kernel"),
+    (50, 140, 4, "yz3_kernel"), (33, 300, 2, "yz3_kernel"), (64, 64, 9, "yz3_kernel"), (65, 128, 8, "yz3_kernel")])
+def test_plane_kernel_of_few_columns(nx, ny, nz, kernel):
+    from paper_2602_12242_gb300 import _lib
+    c = cfg_of(nx=nx, ny=ny, nz=nz, dx=2e-9, dy=2.5e-9, dz=3e-9)
+    h, ctx = field(c)
+    assert (ctx.kernel_name("x_fwd"), ctx.kernel_name("yz_fused")) == ("xfk_kernel", kernel)
+    ref, _ = field(c, demag_path=_lib.MX_DEMAG_GENERIC)
+    assert rel_l2(h, ref) <= TOL
