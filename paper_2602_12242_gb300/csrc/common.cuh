@@ -44,6 +44,16 @@ inline mx_status launch_check(const char* what) {
   return MX_OK;
 }
 
+// The dynamic shared memory a kernel may be launched with.  The limit belongs to the kernel,
+// which every context shares: `bytes` is the most that any of them asks for (cut to a
+// block's), never one context's own need, or the newest context would take it from the others.
+constexpr size_t kMaxSmem = 227 * 1024;
+template <typename K> inline mx_status allow_smem(K kernel, size_t bytes) {
+  MX_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)(bytes < kMaxSmem ? bytes : kMaxSmem)));
+  return MX_OK;
+}
+
 // Programmatic dependent launch.  A kernel launched by launch_pdl may be
 // scheduled while the kernel before it in the stream is still running; it
 // calls pdl_wait() before its first access to memory that kernel writes or

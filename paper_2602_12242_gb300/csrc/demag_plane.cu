@@ -603,8 +603,8 @@ static mx_status yzh_run(mx_ctx* ctx, cudaStream_t st, bool setup) {
   const Grid& g = ctx->g;
   const size_t sm = yzh_smem<E, S>(g.nz);
   if (setup) {
-    if (sm > 227 * 1024) return MX_ERR_UNSUPPORTED;
-    MX_CUDA_TRY(cudaFuncSetAttribute(yzh_kernel<E, S, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    if (sm > kMaxSmem) return MX_ERR_UNSUPPORTED;
+    MX_TRY(allow_smem(yzh_kernel<E, S, P>, yzh_smem<E, S>(P / 2)));
     return MX_OK;
   }
   yzh_kernel<E, S, P><<<2 * g.Hx, kPlaneNT, sm, st>>>(ctx->w1, ctx->w2, g, ctx->nhat, ctx->tw_y, ctx->tw_yh, ctx->tw_z,

@@ -324,8 +324,8 @@ template <int E, int S, int P>
 static mx_status yzq_run(mx_ctx* ctx, cudaStream_t st, bool setup) {
   const size_t sm = yzq_smem<E, S>(ctx->g.nz);
   if (setup) {
-    if (sm > 227 * 1024) return MX_ERR_UNSUPPORTED;
-    MX_CUDA_TRY(cudaFuncSetAttribute(yzq_kernel<E, S, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    if (sm > kMaxSmem) return MX_ERR_UNSUPPORTED;
+    MX_TRY(allow_smem(yzq_kernel<E, S, P>, yzq_smem<E, S>(P / 2)));
     return MX_OK;
   }
   launch_pdl(yzq_kernel<E, S, P>, dim3(4 * ctx->g.Hx), dim3(kQuadNT), sm, st, ctx->w1, ctx->w2, ctx->g, ctx->nhat,

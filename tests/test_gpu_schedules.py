@@ -149,3 +149,20 @@ def test_plane_kernel_of_few_columns(nx, ny, nz, kernel):
     assert (ctx.kernel_name("x_fwd"), ctx.kernel_name("yz_fused")) == ("xfk_kernel", kernel)
     ref, _ = field(c, demag_path=_lib.MX_DEMAG_GENERIC)
     assert rel_l2(h, ref) <= TOL
+
+
+@pytest.mark.parametrize("path,nx,ny,nz,fewer,kernel", [
+    ("MX_DEMAG_AUTO", 40, 512, 16, 9, "yzq_kernel"), ("MX_DEMAG_AUTO", 64, 128, 8, 5, "yzq_kernel"),
+    ("MX_DEMAG_PLANE_PAIR", 64, 200, 4, 3, "yzh_kernel"), ("MX_DEMAG_PLANE", 40, 32, 16, 9, "yzh_kernel")])
+def test_a_newer_context_of_fewer_layers_leaves_the_older_one_usable(path, nx, ny, nz, fewer, kernel):
+    """Both contexts launch the same kernel, the older one with more shared memory."""
+    from paper_2602_12242_gb300 import MX_TERM_DEMAG, _lib
+    from paper_2602_12242_gb300.solver import to_dev4
+    ctx = [None, None]
+    c = cfg_of(nx=nx, ny=ny, nz=nz, dx=2e-9, dy=2.5e-9, dz=3e-9)
+    h, ctx[0] = field(c, demag_path=getattr(_lib, path))
+    _, ctx[1] = field(dict(c, nz=fewer), demag_path=getattr(_lib, path))
+    assert [x.kernel_name("yz_fused") for x in ctx] == [kernel, kernel]
+    again = ctx[0].heff(to_dev4(np.asarray(random_m(c, 41), np.float32)), terms=MX_TERM_DEMAG)
+    ctx[0].sync()
+    assert np.array_equal(again[..., :3].cpu().numpy(), h.astype(np.float32))
