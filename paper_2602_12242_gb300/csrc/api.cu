@@ -114,6 +114,10 @@ static bool row_kernels(const mx_ctx* ctx) { return ctx->xrow && !ctx->plane && 
 // Whether an RK4 or Euler step runs as y/z passes plus one row kernel per stage.
 bool row_steps(const mx_ctx* ctx, int method) { return method != MX_MRI && ctx->p.demag && row_kernels(ctx); }
 
+// Whether a step's stages take the inverse x pass and the local stage as one kernel of the
+// plane path (a learned demag term does not pass through its spectra).
+static bool xlocal_steps(const mx_ctx* ctx) { return ctx->p.demag && ctx->xlocal && !ctx->surrogate && !ctx->fno; }
+
 // The forward x pass of m into w1, which the first row-kernel step of a
 // sequence needs (each later step finds it left by the step before).
 static mx_status lead_x_pass(mx_ctx* ctx, const float4* m, cudaStream_t st) {
@@ -133,7 +137,7 @@ static mx_status enqueue_euler(mx_ctx* ctx, const float4* from, float4* to, doub
     ProfScope ps(ctx, KID_X_INV_LOCAL, st);
     return fast_row_stage(ctx, LM_EULER, io, tail, nullptr, st);
   }
-  if (demag && ctx->xlocal) return plane_stage_xlocal(ctx, LM_EULER, io, st);
+  if (xlocal_steps(ctx)) return plane_stage_xlocal(ctx, LM_EULER, io, st);
   if (demag) MX_TRY(demag_field(ctx, from, hd, st));
   return local_stage(ctx, LM_EULER, io, st);
 }
@@ -147,7 +151,7 @@ static mx_status enqueue_step(mx_ctx* ctx, float4* m, double dt, int method, cud
   if (method == MX_MRI) return mri_step(ctx, m, dt, st);
   const bool demag = ctx->p.demag != 0;
   float4* hd = demag ? ctx->hd : nullptr;
-  const bool xlocal = demag && ctx->xlocal;
+  const bool xlocal = xlocal_steps(ctx);
   if (method == MX_EULER) {
     MX_TRY(enqueue_euler(ctx, m, ctx->sa, dt, st, lead, tail));
     return copy_field(ctx, m, ctx->sa, st);

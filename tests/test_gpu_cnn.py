@@ -192,3 +192,29 @@ def test_tile_walk_matches_oracle(shape, batch):
             n = int(np.prod(s))
             assert rel_l2(g[o:o + n], g_ref.numpy()[o:o + n]) <= 3e-2, s
             o += n
+
+
+@pytest.mark.parametrize("method", ["rk4", "euler"])
+def test_steps_with_a_net_take_its_field_on_every_schedule(method):
+    """A net attached to a context whose own steps fuse the inverse x pass into the local stage: the
+    same kernels as on the plane path, so the same result; and not the FFT's."""
+    from paper_2602_12242_gb300 import _lib
+    from paper_2602_12242_gb300.solver import to_dev4
+    shape = (4, 32, 64)
+    c = cfg_of(nx=64, ny=32, nz=4)
+    net, _ = _net(shape, 1, seed=71)
+    net.set_normalizer(STATS)
+    m0 = _fields(shape, 1, 72)[0]
+    out = {}
+    for path in (_lib.MX_DEMAG_PLANE, _lib.MX_DEMAG_PLANE_XLOCAL):
+        for h in (net.h, None):
+            ctx = context(c, demag_path=path)
+            _lib.mx_set_demag_surrogate(ctx.h, h)
+            m = to_dev4(m0)
+            ctx.rk_step(m, 3, 1e-13, method)
+            ctx.sync()
+            out[path, h is None] = m.clone()
+    plane, xlocal = _lib.MX_DEMAG_PLANE, _lib.MX_DEMAG_PLANE_XLOCAL
+    assert torch.equal(out[plane, False], out[xlocal, False])
+    assert float((out[plane, False] - out[plane, True]).abs().max()) > 1e-4
+    assert float((out[xlocal, True] - out[plane, True]).abs().max()) <= 1e-5
