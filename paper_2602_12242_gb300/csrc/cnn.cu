@@ -435,8 +435,7 @@ __global__ void __launch_bounds__(192, 2)
       mbar_init(&full[q], 1);
       mbar_init(&empty[q], 1);
     }
-    mbar_init(&done, 1);
-    started_s = 0u;
+    mbar_init(&done, 2);  // the MMAs' completion, and the thread that issued them
   }
   if (warp == 1) tmem_alloc(&tbase, W::TCOLS);
   tc_fence_before_sync();
@@ -502,6 +501,8 @@ __global__ void __launch_bounds__(192, 2)
     }
     if (leader) {
       started_s = ok && k > 0 ? 1u : 0u;
+      // (the completion of MMAs does not order this thread's stores; its own arrival does)
+      mbar_arrive(&done);
       tc_commit(&done);
     }
     __syncwarp();
@@ -511,7 +512,7 @@ __global__ void __launch_bounds__(192, 2)
     const int row = 32 * (warp & 3) + lane;
     const bool ok = __all_sync(0xffffffffu, role_wait(&done, 0, flag));
     tc_fence_after_sync();
-    if (ok && *(volatile uint32_t*)&started_s && 32 * (warp & 3) < 3 * CS) {
+    if (ok && started_s && 32 * (warp & 3) < 3 * CS) {
 #pragma unroll 1
       for (int c = 0; c < 3 * CR; c += 8) {
         float v[8];

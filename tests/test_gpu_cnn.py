@@ -218,3 +218,24 @@ def test_steps_with_a_net_take_its_field_on_every_schedule(method):
     assert torch.equal(out[plane, False], out[xlocal, False])
     assert float((out[plane, False] - out[plane, True]).abs().max()) > 1e-4
     assert float((out[xlocal, True] - out[plane, True]).abs().max()) <= 1e-5
+
+
+@pytest.mark.parametrize("shape,batch", [((1, 33, 17), 3), ((2, 17, 33), 3)])
+def test_every_tile_of_the_weight_gradient_arrives(shape, batch):
+    """One tile per block (54 at most per dz; with one layer two thirds of the blocks have none inside the
+    grid): repeated gradients differ by the order of at most 54 FP32 additions per sum (54 x 6e-8), while
+    a block whose sums were left out would change them by about 1 / 54."""
+    from paper_2602_12242_gb300 import _lib
+    net, _ = _net(shape, batch, seed=73)
+    net.set_normalizer(STATS)
+    m = _dev(_fields(shape, batch, 74))
+    tgt = _dev(np.random.default_rng(75).normal(size=(batch,) + shape + (3,)) * 1e5)
+    first = net.loss_grad(m, tgt)[1].double().cpu().numpy()
+    for _ in range(50):
+        g = net.loss_grad(m, tgt)[1].double().cpu().numpy()
+        o = 0
+        for s in ocnn.param_shapes():
+            n = int(np.prod(s))
+            assert rel_l2(g[o:o + n], first[o:o + n]) <= 1e-4, s
+            o += n
+    _lib.mx_cnn_sync(net.h, None)
