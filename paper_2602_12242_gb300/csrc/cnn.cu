@@ -215,6 +215,7 @@ __global__ void __launch_bounds__(ConvTc<CIN, COUT>::threads, 1)
   } else if (warp == 1) {
     {
       // ---- MMA issue: the warp stays together (its operands are uniform), one thread issues
+      pdl_wait();  // (the bounds of its waits do not count the kernel before)
       const uint32_t leader = tc_elect();
       constexpr uint32_t idesc = tc_idesc_bf16(128, NP);
       bool ok = __all_sync(0xffffffffu, role_wait(&wbar, 0, p.flag));
