@@ -315,7 +315,7 @@ typedef struct mx_cnn mx_cnn;
 int mx_cnn_num_params(void);
 
 /* Network for fields of nx*ny*nz cells and batches up to max_batch;
- * allocates all of its buffers (about 15 MB per sample of 64x64x4).  The
+ * allocates all of its buffers (832 bytes per cell of the largest batch).  The
  * parameters start at zero. */
 mx_status mx_cnn_create(mx_cnn **out, int nx, int ny, int nz, int max_batch);
 mx_status mx_cnn_destroy(mx_cnn *net);

@@ -6,12 +6,12 @@
 // solver, per-channel Gaussian normaliser, Adam lr 1e-3, weight decay 1e-4).
 //
 // Activations are BF16 planes of eight channels, [b z][C/8][y][x][8] with C
-// padded to a multiple of 16 (first input: 3 -> 16), and a border of zero cells
-// around every plane (x, y = -1 and up to the tile grid's end) that is written
-// once, at creation.  So every operand tile, halo included, is a set of
-// contiguous rows that bulk copies fetch without a bounds check, and each
-// thread of an epilogue stores 16 bytes next to its neighbour's.  Weights are
-// FP32 masters with BF16 copies in the layout of the tensor cores' operand.
+// padded to a multiple of 16 (first input: 3 -> 16).  An operand tile, halo
+// included, is a box of a tensor map over them: one bulk copy, which fills what
+// leaves the grid with zeros (a step of one cell in x is 16 bytes, the alignment
+// that a copy's start needs).  So nothing but the cells is stored, 832 bytes for
+// each, and each thread of an epilogue stores 16 bytes next to its neighbour's.
+// Weights are FP32 masters with BF16 copies in the layout of the tensor cores' operand.
 //   forward     out = conv(a, W) + b, stored pre-activation y and a = gelu(y)
 //   backward-x  dA_{l-1} = conv(dY_l, W'), W'[tap][ci][co] = W[26 - tap][co][ci],
 //               times gelu'(y_{l-1}) in the epilogue -> dY_{l-1}
@@ -47,13 +47,12 @@ __device__ __forceinline__ float gelu_grad(float y) {
   return 0.5f * (1.f + erff(y * 0.70710678118654752f)) + y * 0.39894228040143268f * expf(-0.5f * y * y);
 }
 
-// Grid and storage of one activation: rows of wq cells, planes of hp rows.
+// Grid and samples of an activation.
 struct ConvDims {
   int nx, ny, nz, batch;
-  int wq, hp;
 };
-// cells from the start of a stored plane to cell (x, y)
-__device__ __forceinline__ long cell_at(const ConvDims& d, int y, int x) { return (long)(y + 1) * d.wq + x + 1; }
+// cells from the start of a plane to cell (x, y)
+__device__ __forceinline__ long cell_at(const ConvDims& d, int y, int x) { return (long)y * d.nx + x; }
 
 // A CTA's tiles [t0, t1): tile t is layer z = t % nz of column t / nz.  The
 // planes z - 1 .. z + 1 inside the grid are loaded once per column (or at the
@@ -203,8 +202,9 @@ __global__ void __launch_bounds__(ConvTc<CIN, COUT>::threads, 1)
           if (seq >= RING) ok = role_wait(&empty[slot], (uint32_t)(seq / RING - 1) & 1u, p.flag);
           if (!ok) break;
           mbar_arrive_expect_tx(&full[slot], T::p_bytes);
-          // (stored cell (y0, x0) is cell (y0 - 1, x0 - 1) of the grid)
-          tensor_load3(smraw + T::w_bytes + slot * T::p_bytes, &in, x0 * 8, y0, (b * d.nz + z) * KC, &full[slot]);
+          // (zeros where the halo leaves the grid)
+          tensor_load3(smraw + T::w_bytes + slot * T::p_bytes, &in, (x0 - 1) * 8, y0 - 1, (b * d.nz + z) * KC,
+                       &full[slot]);
         }
       }
       // no copy is in flight when the block ends (each full barrier's last phase)
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(ConvTc<CIN, COUT>::threads, 1)
     for (int c = 0; c < NH; ++c) bv[c] = (MODE == CM_BWD || cb + c >= COUT || (COUT == 8 && cb + c >= 3)) ? 0.f : __ldg(&p.bias[cb + c]);
     float db[NH] = {};
     double lsum = 0.0;
-    const long plane = (long)d.hp * d.wq * 8;
+    const long plane = (long)d.ny * d.nx * 8;
     // (the walk's divisions once per column: they would be a third of the epilogue's instructions)
     int z = walk.t0 % d.nz, b, y0, x0;
     column(walk.t0 / d.nz, b, y0, x0);
@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(ConvTc<CIN, COUT>::threads, 1)
 // are the longest.
 // Both operands are MN-major (channels contiguous, one 16-byte row of 8 channels
 // per cell, core matrices adjacent along K 128 B apart, 8-channel groups SBO
-// apart): boxes of the stored planes.  Planes of R outside the grid are left out.
+// apart): boxes of the planes.  Planes of R outside the grid are left out.
 // The chains are added in FP32 in ws[(dz 3 + dy) CR + cr][(s, cs)], lanes next to
 // each other.  Bound: the MMAs' operand reads (6 KB per MMA at N = 64) and L2.
 // Measured at 64 samples of 64x64x4, with the kernel before in brackets (a (dz, dy)
@@ -466,10 +466,10 @@ __global__ void __launch_bounds__(192, 2)
         uint64_t* bar = &full[k % ST];
         unsigned char* st = smraw + (k % ST) * W::stage;
         mbar_arrive_expect_tx(bar, W::stage);
-        // S: three copies shifted by -1, 0, +1 in x (stored cell (y + 1, x + 1) is cell (y, x))
+        // S: three copies shifted by -1, 0, +1 in x (zeros outside the grid)
         for (int sh = 0; sh < 3; ++sh)
-          tensor_load3(st + sh * (W::s_bytes / 3), &S, (x0 + sh) * 8, y0 + 1, bz * (CS / 8), bar);
-        tensor_load3(st + W::s_bytes, &R, (x0 + 1) * 8, y0, (bz + dz - 1) * (CR / 8), bar);
+          tensor_load3(st + sh * (W::s_bytes / 3), &S, (x0 + sh - 1) * 8, y0, bz * (CS / 8), bar);
+        tensor_load3(st + W::s_bytes, &R, x0 * 8, y0 - 1, (bz + dz - 1) * (CR / 8), bar);
         ++k;
       }
       // no copy is in flight when the block ends
@@ -567,7 +567,7 @@ __global__ void normalize_in_kernel(const float4* __restrict__ m, bf16_t* __rest
   o.x = pack2((v.x - mean.x) * inv_std.x, (v.y - mean.y) * inv_std.y);
   o.y = pack2((v.z - mean.z) * inv_std.z, 0.f);
   o.z = o.w = 0u;
-  *(uint4*)(x0 + (bz * 2 * d.hp * d.wq + cell_at(d, y, x)) * 8) = o;
+  *(uint4*)(x0 + (bz * 2 * d.ny * d.nx + cell_at(d, y, x)) * 8) = o;
 }
 
 // FP32 master weights -> bf16 [27][CIN_PAD/8][COUT_PAD][8] (forward) and the
@@ -635,7 +635,7 @@ struct mx_cnn {
   bf16_t* wb[4] = {nullptr, nullptr, nullptr, nullptr};
   bf16_t *x0 = nullptr, *a1 = nullptr, *y1 = nullptr, *a2 = nullptr, *y2 = nullptr, *a3 = nullptr, *y3 = nullptr;
   bf16_t *dy4 = nullptr, *dy3 = nullptr, *dy2 = nullptr, *dy1 = nullptr;
-  // the activations as tensors [b z C/8][hp][wq 8] with the boxes of the
+  // the activations as tensors [b z C/8][ny][nx 8] with the boxes of the
   // convolutions' input planes and of the weight gradients' S and R tiles
   CUtensorMap c_x0, c_a1, c_a2, c_a3, c_dy4, c_dy3, c_dy2;
   CUtensorMap s_x0, s_a1, s_dy3, s_dy4, r_dy1, r_dy2, r_a2, r_a3;
@@ -660,16 +660,10 @@ static ConvDims conv_dims(const mx_cnn* n, int batch) {
   d.ny = n->ny;
   d.nz = n->nz;
   d.batch = batch;
-  // the widest tiles are 16 cells in each direction; a border of one cell on each side
-  d.wq = (n->nx + 15) / 16 * 16 + 2;
-  d.hp = (n->ny + 15) / 16 * 16 + 2;
   return d;
 }
-// elements of a stored activation of C channels
-static size_t act_elems(const mx_cnn* n, int C, int batch) {
-  const ConvDims d = conv_dims(n, 1);
-  return (size_t)batch * n->nz * C * d.hp * d.wq;
-}
+// elements of an activation of C channels
+static size_t act_elems(const mx_cnn* n, int C, int batch) { return (size_t)batch * n->cells * C; }
 
 // Tensor map of an activation of C channels, box bx cells x by rows x all C / 8 planes of a layer.
 static mx_status make_map(const mx_cnn* n, CUtensorMap* map, bf16_t* base, int C, int bx, int by) {
@@ -690,9 +684,8 @@ static mx_status make_map(const mx_cnn* n, CUtensorMap* map, bf16_t* base, int C
     set_error("mx_cnn_create: the driver has no cuTensorMapEncodeTiled");
     return MX_ERR_CUDA;
   }
-  const ConvDims d = conv_dims(n, n->max_batch);
-  const cuuint64_t dims[3] = {(cuuint64_t)d.wq * 8, (cuuint64_t)d.hp, (cuuint64_t)n->max_batch * n->nz * (C / 8)};
-  const cuuint64_t strides[2] = {(cuuint64_t)d.wq * 16, (cuuint64_t)d.wq * 16 * d.hp};
+  const cuuint64_t dims[3] = {(cuuint64_t)n->nx * 8, (cuuint64_t)n->ny, (cuuint64_t)n->max_batch * n->nz * (C / 8)};
+  const cuuint64_t strides[2] = {(cuuint64_t)n->nx * 16, (cuuint64_t)n->nx * 16 * n->ny};
   const cuuint32_t box[3] = {(cuuint32_t)bx * 8, (cuuint32_t)by, (cuuint32_t)(C / 8)}, one[3] = {1, 1, 1};
   if (encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -912,10 +905,10 @@ mx_status mx_cnn_create(mx_cnn** out, int nx, int ny, int nz, int max_batch) {
     alloc((void**)&n->wf[l], sizeof(bf16_t) * 27 * kCoutPad[l] * kCinPad[l], true);
     if (l > 0) alloc((void**)&n->wb[l], sizeof(bf16_t) * 27 * bw_in[l] * bw_out[l], true);
   }
-  // zero once: the borders, and the channels that padding adds, are never written
+  // zero once: the channels that padding adds to the sixteen of x0 and dy4 are never written
   bf16_t** act[] = {&n->x0, &n->a1, &n->y1, &n->a2, &n->y2, &n->a3, &n->y3, &n->dy4, &n->dy3, &n->dy2, &n->dy1};
   const int ch[] = {16, 32, 32, 64, 64, 32, 32, 16, 32, 64, 32};
-  for (int q = 0; q < 11; ++q) alloc((void**)act[q], sizeof(bf16_t) * act_elems(n, ch[q], max_batch), true);
+  for (int q = 0; q < 11; ++q) alloc((void**)act[q], sizeof(bf16_t) * act_elems(n, ch[q], max_batch), ch[q] == 16);
   alloc((void**)&n->ws, sizeof(float) * nws, false);
   alloc((void**)&n->loss, sizeof(float), false);
   alloc((void**)&n->flag, sizeof(int), true);

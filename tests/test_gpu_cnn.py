@@ -239,3 +239,18 @@ def test_every_tile_of_the_weight_gradient_arrives(shape, batch):
             assert rel_l2(g[o:o + n], first[o:o + n]) <= 1e-4, s
             o += n
     _lib.mx_cnn_sync(net.h, None)
+
+
+@pytest.mark.parametrize("shape,batch", [((4, 17, 17), 600), ((2, 33, 33), 300), ((1, 700, 1), 900), ((4, 64, 64), 40)])
+def test_memory_follows_the_cells(shape, batch):
+    """416 BF16 channels per cell and nothing for the tiles that a grid does not fill; the other buffers
+    are below 2 MB each, and so is what an allocation is rounded up by (30 buffers in all)."""
+    from paper_2602_12242_gb300.surrogate import Surrogate
+    nz, ny, nx = shape
+    small = Surrogate(8, 8, 1, max_batch=1)  # (the kernels are loaded)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    net = Surrogate(nx, ny, nz, max_batch=batch)
+    used = free - torch.cuda.mem_get_info()[0]
+    assert used <= 832 * nx * ny * nz * batch + 30 * 2 ** 21, used
+    del net, small
