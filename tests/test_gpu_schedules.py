@@ -166,3 +166,21 @@ def test_a_newer_context_of_fewer_layers_leaves_the_older_one_usable(path, nx, n
     again = ctx[0].heff(to_dev4(np.asarray(random_m(c, 41), np.float32)), terms=MX_TERM_DEMAG)
     ctx[0].sync()
     assert np.array_equal(again[..., :3].cpu().numpy(), h.astype(np.float32))
+
+
+@pytest.mark.parametrize("shape,path", [((40, 20, 1), "MX_DEMAG_AUTO"), ((40, 33, 64), "MX_DEMAG_AUTO"),
+                                        ((64, 64, 9), "MX_DEMAG_PLANE"), ((64, 64, 9), "MX_DEMAG_PLANE_XLOCAL")])
+@pytest.mark.parametrize("n", [1, 4, 5])
+def test_profile_times_the_euler_steps_of_a_run(shape, path, n):
+    """The copy that ends a single Euler step is timed for the odd step of a run only, and the profiled
+    steps give the run's bits."""
+    from paper_2602_12242_gb300 import _lib
+    from paper_2602_12242_gb300.solver import to_dev4
+    c = cfg_of(nx=shape[0], ny=shape[1], nz=shape[2], dx=2e-9, dy=2.5e-9, dz=3e-9)
+    ctx = context(c, demag_path=getattr(_lib, path))
+    m0 = np.asarray(random_m(c, 50), np.float32)
+    a, b = to_dev4(m0), to_dev4(m0)
+    ctx.rk_step(a, n, 1e-14, "euler")
+    prof = ctx.profile_step(b, n, 1e-14, "euler")
+    assert prof.get("copy", (0.0, 0))[1] == n % 2
+    assert torch.equal(a, b)
