@@ -1140,16 +1140,16 @@ static FnoOffsets fno_offsets(int K) {
 // tiles, more threads, staged twiddles) where at most one row falls to an SM and
 // its buffers fit.  One field of 160 x 40 takes 72 us with it and 96 without; four
 // fields 138 us with it (two rows on some SMs) and 115 without.
-struct RowShape {
+struct FnoRowShape {
   bool small;
   int threads;
   size_t smem;
 };
 constexpr size_t kFnoMaxSmem = 220 * 1024;
-static RowShape row_shape(const mx_fno* n, int B, bool first) {
+static FnoRowShape row_shape(const mx_fno* n, int B, bool first) {
   const size_t pitch = sizeof(float) * (size_t)fno_pitch(n->wp);
   const size_t bs = first ? 0 : sizeof(float) * (size_t)(kFC + 2 * n->K) * kFC;
-  RowShape r;
+  FnoRowShape r;
   r.smem = bs + (kFC + 2 * n->K) * pitch;
   r.small = (long)B * n->ny <= 152 && r.smem <= kFnoMaxSmem;
   if (!r.small) r.smem = bs + kFC * pitch;
@@ -1194,7 +1194,7 @@ template <bool LIFT>
 static mx_status fno_first(mx_fno* n, const float4* m, float* v, int B, cudaStream_t st) {
   const FnoOffsets f = fno_offsets(n->K);
   const FnoNorm nm = fno_norm(n);
-  const RowShape rs = row_shape(n, B, true);
+  const FnoRowShape rs = row_shape(n, B, true);
   launch_pdl(rs.small ? fno_first_kernel<LIFT, true> : fno_first_kernel<LIFT, false>, dim3((unsigned)(B * n->ny)),
              dim3(rs.threads), rs.smem, st, m, nm.mean, nm.inv_std, n->params + f.P, n->params + f.p, v, n->A, n->nx,
              n->wp, n->K, n->twx);
@@ -1205,7 +1205,7 @@ template <bool BWD>
 static mx_status fno_row(mx_fno* n, int l, const float* vin, float* pre, float* out, const float* gpre, bool gelu_out,
                          bool next, int B, cudaStream_t st) {
   const FnoOffsets f = fno_offsets(n->K);
-  const RowShape rs = row_shape(n, B, false);
+  const FnoRowShape rs = row_shape(n, B, false);
   const float scale = 1.f / ((float)n->ny * (float)n->nx);
   launch_pdl(rs.small ? fno_row_kernel<BWD, 4> : fno_row_kernel<BWD, 8>, dim3((unsigned)(B * n->ny)),
              dim3(rs.threads), rs.smem, st, n->A, vin, n->params + f.W[l], BWD ? nullptr : n->params + f.w[l], pre, out, gpre, n->nx, n->wp, n->K,
