@@ -380,12 +380,12 @@ struct AdjRowLaunch {
     const dim3 grid((g.ny * g.nz + R - 1) / R);
     if (begin) {
       auto k = c.dmi ? adj_row_begin_kernel<M, R, NT, true> : adj_row_begin_kernel<M, R, NT, false>;
-      RowShape<M, R>::allow(k);
+      MX_TRY((RowShape<M, R>::allow(k)));
       launch_pdl(k, grid, dim3(NT), RowShape<M, R>::smem, st, ctx->w1, g, ctx->tw_m, ctx->tw_x, *a, c, dt);
       return launch_check("adj_row_begin_kernel");
     }
     auto k = c.dmi ? adj_row_kernel<M, R, NT, true> : adj_row_kernel<M, R, NT, false>;
-    RowShape<M, R>::allow(k);
+    MX_TRY((RowShape<M, R>::allow(k)));
     launch_pdl(k, grid, dim3(NT), RowShape<M, R>::smem, st, ctx->w1, g, ctx->tw_m, ctx->tw_x, *a, c, dt, stage,
                chain ? 1 : 0);
     return launch_check("adj_row_kernel");

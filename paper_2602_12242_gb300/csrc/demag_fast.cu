@@ -575,7 +575,7 @@ mx_status yz2d_pass(mx_ctx* ctx, cudaStream_t st) { return yz2d_dispatch(ctx, st
 template <int M, int R, int NT>
 static mx_status run_xf(mx_ctx* ctx, const float4* m, cudaStream_t st) {
   const Grid& g = ctx->g;
-  RowShape<M, R>::allow(xf_kernel<M, R, NT>);
+  MX_TRY((RowShape<M, R>::allow(xf_kernel<M, R, NT>)));
   launch_pdl(xf_kernel<M, R, NT>, dim3((g.ny * g.nz + R - 1) / R), dim3(NT), RowShape<M, R>::smem, st, m, g,
              (float)ctx->p.Ms, ctx->ms_map, ctx->w1, ctx->tw_m, ctx->tw_x);
   return launch_check("xf_kernel");
@@ -584,7 +584,7 @@ static mx_status run_xf(mx_ctx* ctx, const float4* m, cudaStream_t st) {
 template <int M, int R, int NT>
 static mx_status run_xi(mx_ctx* ctx, float4* hd, cudaStream_t st) {
   const Grid& g = ctx->g;
-  RowShape<M, R>::allow(xi_kernel<M, R, NT>);
+  MX_TRY((RowShape<M, R>::allow(xi_kernel<M, R, NT>)));
   launch_pdl(xi_kernel<M, R, NT>, dim3((g.ny * g.nz + R - 1) / R), dim3(NT), RowShape<M, R>::smem, st, ctx->w1, g, hd,
              ctx->tw_m, ctx->tw_x);
   return launch_check("xi_kernel");
@@ -596,7 +596,7 @@ static mx_status run_xr(mx_ctx* ctx, int mode, const StageIO& io, bool xf_next, 
   const LocalCoef c = local_coef(ctx);
   auto k = mode == LM_HEFF ? (c.dmi ? xr_kernel<M, R, NT, true, true> : xr_kernel<M, R, NT, false, true>)
                            : (c.dmi ? xr_kernel<M, R, NT, true, false> : xr_kernel<M, R, NT, false, false>);
-  RowShape<M, R>::allow(k);
+  MX_TRY((RowShape<M, R>::allow(k)));
   launch_pdl(k, dim3((g.ny * g.nz + R - 1) / R), dim3(NT), RowShape<M, R>::smem, st, ctx->w1, g, ctx->tw_m, ctx->tw_x, io, c, mode, xf_next ? 1 : 0, hd_out,
              ctx->flag);
   return launch_check("xr_kernel");

@@ -108,9 +108,10 @@ template <int M, int R> struct RowShape {
   static constexpr int lines = NF / L::TL;
   static constexpr int half = lines * L::PITCH;  // float2 of one half of the buffer
   static constexpr size_t smem = sizeof(float2) * 2 * half;
+  static_assert(smem <= kMaxSmem, "row kernel shared memory");
   // (called before a launch of a kernel with these blocks; only M = 1024 needs it)
-  template <typename K> static void allow(K kernel) {
-    if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  template <typename K> static mx_status allow(K kernel) {
+    return smem > 48 * 1024 ? allow_smem(kernel, smem) : MX_OK;
   }
   // The buffer half that the inverse rows are left in and the forward rows are
   // read from: after an inverse's exchanges the next half in turn, and the one after that.
