@@ -22,7 +22,7 @@ __global__ void __launch_bounds__(NT) xf_kernel(const float4* __restrict__ m, Gr
   RowTw<M> tw;
   tw.load(twM, twP);
   pdl_wait_next();
-  xf_stage<M, R, NT, false>(sm, m, g, ms, ms_map, blockIdx.x * R);
+  xf_stage<M, R, NT>(sm, m, g, ms, ms_map, blockIdx.x * R);
   xf_rows<M, R>(sm, g, w1, blockIdx.x * R, tw);
 }
 

@@ -241,7 +241,7 @@ static mx_status yz3_pz(mx_ctx* ctx, bool km, cudaStream_t st, bool setup) {
 mx_status yz3_pass(mx_ctx* ctx, bool km, cudaStream_t st, bool setup) {
   if (setup) MX_TRY(upload_w32());
   switch (ctx->g.Py / 2) {
-    case 512: return yz3_pz<32, 16, true, false>(ctx, km, st, setup);
+    case 512: return yz3_pz<32, 16, false, false>(ctx, km, st, setup);  // (five layers take 143 KB)
     case 256: return yz3_pz<16, 16, true, false>(ctx, km, st, setup);
     case 128: return yz3_pz<16, 8, true, false>(ctx, km, st, setup);
     case 64: return yz3_pz<8, 8, true, true>(ctx, km, st, setup);

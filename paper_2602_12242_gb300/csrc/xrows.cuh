@@ -190,7 +190,7 @@ __device__ __forceinline__ void xf_cell(float2* sm, int r, int i, float3 v) {
 }
 
 // xf_cell for the cells of rows row0 .. row0 + R - 1 of Ms m in global memory.
-template <int M, int R, int NT, bool COHERENT>
+template <int M, int R, int NT>
 __device__ __forceinline__ void xf_stage(float2* sm, const float4* __restrict__ m, const Grid& g, float ms,
                                          const float* __restrict__ ms_map, int row0) {
   const int total = min(R, g.ny * g.nz - row0) * g.nx;
@@ -198,7 +198,7 @@ __device__ __forceinline__ void xf_stage(float2* sm, const float4* __restrict__ 
   for (int e = threadIdx.x; e < total; e += NT) {
     const int r = R == 1 ? 0 : e / g.nx, i = e - r * g.nx;
     const long idx = (long)row0 * g.nx + e;
-    const float4 a = COHERENT ? m[idx] : __ldg(&m[idx]);
+    const float4 a = __ldg(&m[idx]);
     const float s = ms_map ? __ldg(&ms_map[idx]) : ms;
     xf_cell<M, R>(sm, r, i, make_float3(s * a.x, s * a.y, s * a.z));
   }
