@@ -227,3 +227,23 @@ def test_adjoint_workload_full_2000_steps():
     a checkpoint every 100 (about 30 CPU minutes)."""
     c, Ms, m0, patch, g, gms = _workload(2000, 100)
     _check_against_oracle(c, Ms, m0, patch, g, gms, 2000, 2)
+
+
+@pytest.mark.parametrize("shape", [(1, 11, 40), (2, 9, 100), (1, 10, 200), (1, 11, 300), (2, 9, 600), (1, 12, 1000)])
+def test_adjoint_row_kernels_of_every_row_length(shape):
+    """Rows of 40 to 1000 cells (Px/2 = 64 .. 1024; from 257 cells on a thread has two or three of them),
+    ragged, with a last block of part of its rows, DMI, anisotropy and an Ms map: a few steps across a
+    checkpoint against the oracle's discrete adjoint."""
+    nz, ny, nx = shape
+    rng = np.random.default_rng(36)
+    c = cfg_of(nx=nx, ny=ny, nz=nz, D=1e-3, dmi=True, Ku=2e4, ku_axis=(0.1, 0.4, 1.0), alpha=0.25,
+               h_bias=(1e4, 0.0, 4e4))
+    Ms = f32(rng.uniform(6e5, 1e6, size=shape))
+    m0 = f32(rng.normal(size=shape + (3,)))
+    patch = ((2, ny - 1), (3, nx - 2))
+    ctx, _, g, gms = run_case(c, Ms, m0, 5, 3, patch, 1e-14)
+    assert ctx.kernel_name("x_inv_local") == "xr_kernel"
+    p = problem(c, Ms=Ms)
+    _, g_ref, gms_ref = oadj.gradient(p, m0, 1e-14, 5, lambda m: oadj.patch_mean_mz(m, patch))
+    assert rel_l2(g, g_ref.numpy()) <= TOL_GRAD, rel_l2(g, g_ref.numpy())
+    assert rel_l2(gms, gms_ref.numpy()) <= TOL_GRAD, rel_l2(gms, gms_ref.numpy())

@@ -26,7 +26,7 @@ def field(c, **kw):
     return h, ctx
 
 
-# (nx, ny, nz): Py/2 = 16 .. 512 with Pz = 4 .. 32, full and ragged nz <= Pz/2 and ny <= Py/2,
+# (nx, ny, nz): Py/2 = 16 .. 256 with Pz = 4 .. 32, full and ragged nz <= Pz/2 and ny <= Py/2,
 # one and two kx columns per block (Hx above and below 608), an odd last column
 FEW_LAYERS = [(40, 9, 2), (33, 16, 16), (20, 13, 9), (64, 32, 16), (37, 21, 5), (30, 17, 13), (50, 64, 8), (40, 40, 4),
               (41, 33, 2), (70, 128, 5), (24, 100, 4), (30, 77, 2), (20, 65, 7), (24, 256, 2), (600, 24, 2),
@@ -80,7 +80,7 @@ def test_many_row_x_kernels_match_generic_passes(shape, ms_map):
     assert rel_l2(h, ref) <= TOL
 
 
-# (nx, ny): one layer, Px/2 and Py/2 = 16 .. 1024 and 16 .. 512, one, two, four and eight columns per
+# (nx, ny): one layer, Px/2 and Py/2 = 16 .. 1024 and 16 .. 512, one, two and four columns per
 # block and the wide kernel, odd last columns, ragged rows
 FILMS = [(9, 9), (16, 16), (31, 30), (70, 20), (640, 30), (33, 33), (200, 60), (700, 50), (100, 100), (300, 128),
          (1000, 70), (60, 200), (200, 150), (300, 200), (120, 300), (130, 500)]
@@ -184,3 +184,35 @@ def test_profile_times_the_euler_steps_of_a_run(shape, path, n):
     prof = ctx.profile_step(b, n, 1e-14, "euler")
     assert prof.get("copy", (0.0, 0))[1] == n % 2
     assert torch.equal(a, b)
+
+
+# (nx, ny, nz, kx-major): every (Py/2, Pz) that the few-layer kernel runs on the plane path's layout, and
+# those of long columns and of two kx columns per block (Hx > 608) in place
+@pytest.mark.parametrize("nx,ny,nz,km", [
+    (100, 50, 14, True), (64, 64, 16, True), (100, 128, 8, True), (40, 150, 4, True), (100, 256, 3, True),
+    (100, 150, 6, True), (70, 256, 8, True), (40, 300, 2, True), (100, 512, 2, True), (100, 280, 3, True),
+    (20, 50, 14, False), (30, 100, 7, False), (20, 200, 4, False), (24, 256, 3, False), (20, 150, 6, False),
+    (24, 256, 8, False), (20, 300, 2, False), (24, 512, 2, False), (20, 280, 3, False),
+    (1000, 60, 4, False), (600, 100, 3, False), (600, 200, 2, False), (600, 60, 7, False), (600, 30, 14, False),
+    (1000, 12, 15, False), (520, 9, 7, False)])
+def test_few_layer_kernel_of_every_layout_matches_generic_passes(nx, ny, nz, km):
+    from paper_2602_12242_gb300 import _lib
+    c = cfg_of(nx=nx, ny=ny, nz=nz, dx=2e-9, dy=2.5e-9, dz=3e-9)
+    h, ctx = field(c)
+    assert ctx.kernel_name("yz_fused") == "yz3_kernel"
+    assert (ctx.kernel_name("x_fwd") == "xfk_kernel") == km
+    ref, _ = field(c, demag_path=_lib.MX_DEMAG_GENERIC)
+    assert rel_l2(h, ref) <= TOL
+
+
+# films of 2049 kx columns: eight columns per block (rows of up to 64), four, and the wide kernel, after the
+# size-generic x passes
+@pytest.mark.parametrize("nx,ny", [(1025, 16), (1300, 9), (1100, 30), (1025, 60), (1100, 100), (1030, 130), (1025, 257)])
+def test_film_kernels_of_many_columns_match_generic_passes(nx, ny):
+    from paper_2602_12242_gb300 import _lib
+    c = cfg_of(nx=nx, ny=ny, nz=1, dx=2e-9, dy=2.5e-9, dz=3e-9)
+    h, ctx = field(c)
+    assert ctx.padded_dims[0] == 4096 and ctx.kernel_name("x_fwd") == "x_fwd_kernel"
+    assert ctx.kernel_name("yz_fused") == ("yz2d_wide_kernel" if ny > 128 else "yz2d_kernel")
+    ref, _ = field(c, demag_path=_lib.MX_DEMAG_GENERIC)
+    assert rel_l2(h, ref) <= TOL
