@@ -78,7 +78,7 @@ struct PrepIn {
   __device__ __forceinline__ void load(const float4* __restrict__ mf, const float4* __restrict__ hdf, const Grid& g,
                                        const LocalCoef& c, int i, int j, int k, long idx) {
     m = f3(mf[idx]);
-    hd = hdf ? f3(__ldg(&hdf[idx])) : make_float3(0.f, 0.f, 0.f);
+    hd = hdf ? f3(hdf[idx]) : make_float3(0.f, 0.f, 0.f);
     e = easy_axis(c, idx);
     ms = c.ms_map ? __ldg(&c.ms_map[idx]) : c.Ms;
     cK = aniso_coef(c, idx);
@@ -192,7 +192,7 @@ __device__ __forceinline__ float3 finish_cell(const float4* __restrict__ m, cons
                                               int i, int j, int k, long idx) {
   FinishIn in;
   in.load(m, wbuf, gm, lam_u4, lam_acc, dms, g, c, i, j, k, idx, STAGE);
-  return finish_apply<DMI>(in, hdw ? f3(__ldg(&hdw[idx])) : make_float3(0.f, 0.f, 0.f), lam_acc, dms, c, dt, idx, STAGE);
+  return finish_apply<DMI>(in, hdw ? f3(hdw[idx]) : make_float3(0.f, 0.f, 0.f), lam_acc, dms, c, dt, idx, STAGE);
 }
 
 template <bool DMI>

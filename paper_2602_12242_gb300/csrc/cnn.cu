@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(ConvTc<CIN, COUT>::threads, 1)
           p.field[cell] = make_float4(q[0] * p.sd.x + p.mean.x, q[1] * p.sd.y + p.mean.y, q[2] * p.sd.z + p.mean.z, 0.f);
         } else {
           // SmoothL1 (beta 1) against the normalised target
-          const float4 tg = __ldg(&p.target[cell]);
+          const float4 tg = p.target[cell];
           const float e[3] = {q[0] - (tg.x - p.mean.x) * p.sd.x, q[1] - (tg.y - p.mean.y) * p.sd.y,
                               q[2] - (tg.z - p.mean.z) * p.sd.z};
           float g[3], l = 0.f;
@@ -542,7 +542,7 @@ struct WgradOut {
 struct WgradOuts {
   WgradOut l[4];
 };
-__global__ void wgrad_finish_kernel(const float* __restrict__ ws, float* __restrict__ grad, WgradOuts o) {
+__global__ void wgrad_finish_kernel(const float* ws, float* __restrict__ grad, WgradOuts o) {
   const WgradOut l = o.l[blockIdx.y];
   pdl_wait_next();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -555,7 +555,7 @@ __global__ void wgrad_finish_kernel(const float* __restrict__ ws, float* __restr
 }
 
 // input normalisation: m float4 -> the first eight channels of the padded input
-__global__ void normalize_in_kernel(const float4* __restrict__ m, bf16_t* __restrict__ x0, ConvDims d, long ncells,
+__global__ void normalize_in_kernel(const float4* m, bf16_t* __restrict__ x0, ConvDims d, long ncells,
                                     float3 mean, float3 inv_std) {
   const long c = (long)blockIdx.x * blockDim.x + threadIdx.x;
   pdl_wait_next();

@@ -59,6 +59,13 @@ template <typename K> inline mx_status allow_smem(K kernel, size_t bytes) {
 // calls pdl_wait() before its first access to memory that kernel writes or
 // reads (the wait returns once that kernel has completed and its writes are
 // visible; without a programmatic dependency it returns at once).
+//
+// What such a kernel reads of the kernels before it goes through plain loads: no
+// __ldg and no `const __restrict__` kernel parameter.  Those are non-coherent loads,
+// which the compiler takes for constants and may move above the wait (memory clobber
+// or not).  deep_yf_kernel did so behind row kernels of at most a block per SM: a deep
+// grid of 26x25x20 cells took the spectrum of the stage before.  Both are for tables,
+// parameters and maps that no kernel of the chain writes.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // pdl_wait_next: after the wait, a grid of at most a block per SM lets the next

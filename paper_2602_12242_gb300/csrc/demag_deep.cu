@@ -135,7 +135,7 @@ template <int L> struct Deep {
 // ---------------------------------------------------------------------------
 template <int L>
 __global__ void __launch_bounds__(Deep<L>::NT)
-    deep_yf_kernel(const float2* __restrict__ w1, float2* __restrict__ w2, Grid g, const float2* __restrict__ twP) {
+    deep_yf_kernel(const float2* w1, float2* w2, Grid g, const float2* __restrict__ twP) {
   typedef Deep<L> D;
   constexpr int E = D::E, S = D::S, T = D::T;
   extern __shared__ __align__(16) float2 sm[];
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(Deep<L>::NT)
 #pragma unroll
   for (int n = 0; n < E; ++n) {
     const int y = s + S * n;
-    v[n] = ok && y < g.ny ? __ldg(&src[(long)y * g.Hx]) : make_float2(0.f, 0.f);
+    v[n] = ok && y < g.ny ? src[(long)y * g.Hx] : make_float2(0.f, 0.f);
   }
   __syncthreads();  // the table
   float2* line = sm + D::TW + (h * T + t) * D::PITCH;
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(Deep<L>::NT)
 
 template <int L>
 __global__ void __launch_bounds__(Deep<L>::NT)
-    deep_yi_kernel(const float2* __restrict__ w2, float2* __restrict__ w1, Grid g, const float2* __restrict__ twP) {
+    deep_yi_kernel(const float2* w2, float2* w1, Grid g, const float2* __restrict__ twP) {
   typedef Deep<L> D;
   constexpr int E = D::E, S = D::S, T = D::T;
   extern __shared__ __align__(16) float2 sm[];
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(Deep<L>::NT)
   for (int j = 0; j < D::J; ++j)
 #pragma unroll
     for (int q = 0; q < S; ++q)
-      v[j * S + q] = ok ? __ldg(&src[(long)(2 * (s + S * j + E * q) + h) * g.Hx]) : make_float2(0.f, 0.f);
+      v[j * S + q] = ok ? src[(long)(2 * (s + S * j + E * q) + h) * g.Hx] : make_float2(0.f, 0.f);
   __syncthreads();
   float2* line = sm + D::TW + (h * T + t) * D::PITCH;
   D::inv1(v, line, s, h, sm);

@@ -15,7 +15,7 @@
 namespace mx {
 
 template <int M, int R, int NT>
-__global__ void __launch_bounds__(NT) xf_kernel(const float4* __restrict__ m, Grid g, float ms,
+__global__ void __launch_bounds__(NT) xf_kernel(const float4* m, Grid g, float ms,
                                                 const float* __restrict__ ms_map, float2* __restrict__ w1,
                                                 const float2* __restrict__ twM, const float2* __restrict__ twP) {
   extern __shared__ float2 sm[];
@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(NT) xf_kernel(const float4* __restrict__ m, Gr
 // x inverse (c2r).
 // ---------------------------------------------------------------------------
 template <int M, int R, int NT>
-__global__ void __launch_bounds__(NT) xi_kernel(const float2* __restrict__ w1, Grid g, float4* __restrict__ hd,
+__global__ void __launch_bounds__(NT) xi_kernel(const float2* w1, Grid g, float4* __restrict__ hd,
                                                 const float2* __restrict__ twM, const float2* __restrict__ twP) {
   extern __shared__ float2 sm[];
   const int row0 = blockIdx.x * R;
@@ -62,7 +62,7 @@ template <int E, int S, int R> struct ManyRows {
 };
 
 template <int E, int S, int R>
-__global__ void __launch_bounds__(3 * R * S) xf_many_kernel(const float4* __restrict__ m, Grid g, float ms,
+__global__ void __launch_bounds__(3 * R * S) xf_many_kernel(const float4* m, Grid g, float ms,
                                                            const float* __restrict__ ms_map, float2* __restrict__ w1,
                                                            const float2* __restrict__ twM,
                                                            const float2* __restrict__ twP) {
@@ -83,8 +83,8 @@ __global__ void __launch_bounds__(3 * R * S) xf_many_kernel(const float4* __rest
     const int r = e / HALF, i = 2 * (e % HALF);
     const bool in = e < R * HALF && row0 + r < nrows;
     const long cell = (long)(row0 + r) * g.nx + i;
-    va[j] = in && i < g.nx ? __ldg(&m[cell]) : make_float4(0.f, 0.f, 0.f, 0.f);
-    vb[j] = in && i + 1 < g.nx ? __ldg(&m[cell + 1]) : make_float4(0.f, 0.f, 0.f, 0.f);
+    va[j] = in && i < g.nx ? m[cell] : make_float4(0.f, 0.f, 0.f, 0.f);
+    vb[j] = in && i + 1 < g.nx ? m[cell + 1] : make_float4(0.f, 0.f, 0.f, 0.f);
     sa[j] = sb[j] = ms;
     if (ms_map) {
       if (in && i < g.nx) sa[j] = __ldg(&ms_map[cell]);
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(3 * R * S) xf_many_kernel(const float4* __rest
 }
 
 template <int E, int S, int R>
-__global__ void __launch_bounds__(3 * R * S) xi_many_kernel(const float2* __restrict__ w1, Grid g,
+__global__ void __launch_bounds__(3 * R * S) xi_many_kernel(const float2* w1, Grid g,
                                                            float4* __restrict__ hd, const float2* __restrict__ twM,
                                                            const float2* __restrict__ twP) {
   typedef BankLine<E, S> BL;
@@ -153,8 +153,8 @@ __global__ void __launch_bounds__(3 * R * S) xi_many_kernel(const float2* __rest
       a[u] = b[u] = make_float2(0.f, 0.f);
       if (e < NE && row < nrows) {
         const float2* X = w1 + (line % 3) * cs + (long)row * g.Hx;
-        a[u] = __ldg(&X[k]);
-        b[u] = cconj(__ldg(&X[M - k]));
+        a[u] = X[k];
+        b[u] = cconj(X[M - k]);
       }
     }
 #pragma unroll

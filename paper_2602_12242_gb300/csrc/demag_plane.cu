@@ -49,7 +49,7 @@ template <int E, int S> struct YzhPitch {
 // x forward into the kx-major spectrum.
 // ---------------------------------------------------------------------------
 template <int E, int S>
-__global__ void __launch_bounds__(3 * kRows * S, S >= 32 ? 1 : 2) xfk_kernel(const float4* __restrict__ m, Grid g, float ms,
+__global__ void __launch_bounds__(3 * kRows * S, S >= 32 ? 1 : 2) xfk_kernel(const float4* m, Grid g, float ms,
                                                             const float* __restrict__ ms_map, float2* __restrict__ w1,
                                                             const float2* __restrict__ twM,
                                                             const float2* __restrict__ twP) {
@@ -79,8 +79,8 @@ __global__ void __launch_bounds__(3 * kRows * S, S >= 32 ? 1 : 2) xfk_kernel(con
         const int y = y0 + r;
         const bool in = e < kRows * HALF && y < g.ny;
         const long cell = ((long)z * g.ny + (in ? y : 0)) * g.nx + 2 * n;
-        va[j] = (in && 2 * n < g.nx) ? __ldg(&m[cell]) : make_float4(0.f, 0.f, 0.f, 0.f);
-        vb[j] = (in && 2 * n + 1 < g.nx) ? __ldg(&m[cell + 1]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        va[j] = (in && 2 * n < g.nx) ? m[cell] : make_float4(0.f, 0.f, 0.f, 0.f);
+        vb[j] = (in && 2 * n + 1 < g.nx) ? m[cell + 1] : make_float4(0.f, 0.f, 0.f, 0.f);
       }
     }
     const int z = b / ychunks, y0 = (b % ychunks) * kRows;
@@ -205,8 +205,8 @@ __device__ __forceinline__ void xik_lines(float2* sm, const float2* __restrict__
         const int k = k0 + KS * (j0 + u);
         a[u] = b[u] = make_float2(0.f, 0.f);
         if (j0 + u < J && k <= M / 2 && y < g.ny) {
-          a[u] = __ldg(&src[(long)k * plane]);
-          b[u] = cconj(__ldg(&src[(long)(M - k) * plane]));
+          a[u] = src[(long)k * plane];
+          b[u] = cconj(src[(long)(M - k) * plane]);
         }
       }
 #pragma unroll
@@ -226,7 +226,7 @@ __device__ __forceinline__ void xik_lines(float2* sm, const float2* __restrict__
 }
 
 template <int E, int S>
-__global__ void __launch_bounds__(3 * kRows * S, S >= 32 ? 1 : 2) xik_kernel(const float2* __restrict__ w2, Grid g,
+__global__ void __launch_bounds__(3 * kRows * S, S >= 32 ? 1 : 2) xik_kernel(const float2* w2, Grid g,
                                                             float4* __restrict__ hd, const float2* __restrict__ twM,
                                                             const float2* __restrict__ twP) {
   constexpr int M = E * S;
@@ -271,7 +271,7 @@ __device__ __forceinline__ void xil_cells(const float2* sm, int P, int NT, const
 }
 
 template <int E, int S, bool DMI>
-__global__ void __launch_bounds__(3 * kRows * S, S >= 32 ? 1 : 2) xil_kernel(const float2* __restrict__ w2, Grid g,
+__global__ void __launch_bounds__(3 * kRows * S, S >= 32 ? 1 : 2) xil_kernel(const float2* w2, Grid g,
                                                             const float2* __restrict__ twM,
                                                             const float2* __restrict__ twP, StageIO io, LocalCoef c,
                                                             int mode, int* flag) {

@@ -82,7 +82,7 @@ __device__ __forceinline__ void named_sync(int id, int count) {
 
 template <int E, int S, int P>
 __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kQuadNT, 2)
-    yzq_kernel(const float2* __restrict__ w1, float2* __restrict__ w2, Grid g, const float* __restrict__ nhk,
+    yzq_kernel(const float2* w1, float2* __restrict__ w2, Grid g, const float* __restrict__ nhk,
                const float2* __restrict__ twPy) {
   constexpr int L4 = E * S;
   constexpr int PITCH = LineFft<E, S>::kPitch;
@@ -130,8 +130,8 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kQuadNT, 2)
         const int e = base + tid + u * NT;
         const int line = lb + e / L4, y = e % L4;
         const float2* src = w1 + kxoff + (long)line * ny;
-        a[u] = (e < cnt && y < ny) ? __ldg(src + y) : make_float2(0.f, 0.f);
-        b[u] = (e < cnt && y + L4 < ny) ? __ldg(src + y + L4) : make_float2(0.f, 0.f);
+        a[u] = (e < cnt && y < ny) ? src[y] : make_float2(0.f, 0.f);
+        b[u] = (e < cnt && y + L4 < ny) ? src[y + L4] : make_float2(0.f, 0.f);
       }
       if (base == 0) cluster_wait();  // every CTA of the cluster has started
       float2* dst0 = const_cast<float2*>(cluster_map(plane, 0u));

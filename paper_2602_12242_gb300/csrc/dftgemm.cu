@@ -151,7 +151,7 @@ __device__ __forceinline__ void dft_stage1(float2* lines, unsigned char* sa, uns
 }
 
 template <int S>
-__global__ void __launch_bounds__(DftShape<S>::NT) xfk_dft_kernel(const float4* __restrict__ m, Grid g, float ms,
+__global__ void __launch_bounds__(DftShape<S>::NT) xfk_dft_kernel(const float4* m, Grid g, float ms,
                                                                   const float* __restrict__ ms_map,
                                                                   float2* __restrict__ w1, const bf16_t* __restrict__ agl,
                                                                   const float2* __restrict__ twM,
@@ -179,12 +179,12 @@ __global__ void __launch_bounds__(DftShape<S>::NT) xfk_dft_kernel(const float4* 
       const long cell = ((long)z * g.ny + y) * g.nx;
       const int i0 = 2 * n, i1 = i0 + 1;
       if (i0 < g.nx) {
-        const float4 a = __ldg(&m[cell + i0]);
+        const float4 a = m[cell + i0];
         const float s = ms_map ? __ldg(&ms_map[cell + i0]) : ms;
         zx.x = s * a.x; zy.x = s * a.y; zz.x = s * a.z;
       }
       if (i1 < g.nx) {
-        const float4 b = __ldg(&m[cell + i1]);
+        const float4 b = m[cell + i1];
         const float s = ms_map ? __ldg(&ms_map[cell + i1]) : ms;
         zx.y = s * b.x; zy.y = s * b.y; zz.y = s * b.z;
       }
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(DftShape<S>::NT) xfk_dft_kernel(const float4* 
 }
 
 template <int S>
-__global__ void __launch_bounds__(DftShape<S>::NT) xik_dft_kernel(const float2* __restrict__ w2, Grid g,
+__global__ void __launch_bounds__(DftShape<S>::NT) xik_dft_kernel(const float2* w2, Grid g,
                                                                   float4* __restrict__ hd, const bf16_t* __restrict__ agl,
                                                                   const float2* __restrict__ twM,
                                                                   const float2* __restrict__ twP, int* flag) {
@@ -250,8 +250,8 @@ __global__ void __launch_bounds__(DftShape<S>::NT) xik_dft_kernel(const float2* 
     float2 v = make_float2(0.f, 0.f);
     if (y < g.ny) {
       const long o = ((long)c * g.nz + z) * g.ny + y;
-      const float2 a = __ldg(&w2[(long)k * plane + o]);
-      const float2 b = cconj(__ldg(&w2[(long)(M - k) * plane + o]));
+      const float2 a = w2[(long)k * plane + o];
+      const float2 b = cconj(w2[(long)(M - k) * plane + o]);
       const float2 Sv = cadd(a, b);
       const float2 t = cmul(cconj(__ldg(&twP[k])), csub(a, b));
       v = make_float2(Sv.x - t.y, Sv.y + t.x);

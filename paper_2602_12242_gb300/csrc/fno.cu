@@ -174,8 +174,8 @@ __device__ __forceinline__ void fno_copy_row(float* vs, const float* v, int Wp, 
 // stored, and its row DFT.  Otherwise the row DFT of the stored row v.
 template <bool LIFT, bool SMALL>
 __global__ void __launch_bounds__(SMALL ? 384 : 128)
-    fno_first_kernel(const float4* __restrict__ m, float3 mean, float3 inv_std, const float* __restrict__ Pw,
-                     const float* __restrict__ pb, float* __restrict__ v, float2* __restrict__ A, int W, int Wp, int K,
+    fno_first_kernel(const float4* m, float3 mean, float3 inv_std, const float* Pw,
+                     const float* pb, float* __restrict__ v, float2* __restrict__ A, int W, int Wp, int K,
                      const float* __restrict__ tw) {
   extern __shared__ __align__(16) float fsm[];
   const int P = fno_pitch(Wp);
@@ -191,16 +191,14 @@ __global__ void __launch_bounds__(SMALL ? 384 : 128)
       float nx = 0.f, ny = 0.f, nz = 0.f;
       const bool in = x < W;
       if (in) {
-        const float4 a = __ldg(&m[r * W + x]);
+        const float4 a = m[r * W + x];
         nx = (a.x - mean.x) * inv_std.x;
         ny = (a.y - mean.y) * inv_std.y;
         nz = (a.z - mean.z) * inv_std.z;
       }
 #pragma unroll
       for (int c = c0; c < c0 + 8; ++c) {
-        const float o = in ? __ldg(&pb[c]) + __ldg(&Pw[c * 3]) * nx + __ldg(&Pw[c * 3 + 1]) * ny +
-                                 __ldg(&Pw[c * 3 + 2]) * nz
-                           : 0.f;
+        const float o = in ? pb[c] + Pw[c * 3] * nx + Pw[c * 3 + 1] * ny + Pw[c * 3 + 2] * nz : 0.f;
         vs[c * P + x] = o;
         row[(long)c * Wp + x] = o;
       }
@@ -375,7 +373,7 @@ __global__ void __cluster_dims__(kMidCl, 1, 1) __launch_bounds__(kMidWarps * 32)
 // Forward column DFT: thread (c) of column (b, kx) sums kMidM modes over all rows,
 // eight rows' values in flight; the block's twiddles in shared memory by chunks of rows.
 constexpr int kMidM = 8, kMidY = 8;
-__global__ void __launch_bounds__(128) fno_dft_y_kernel(const float2* __restrict__ A, float2* __restrict__ X, int B,
+__global__ void __launch_bounds__(128) fno_dft_y_kernel(const float2* A, float2* __restrict__ X, int B,
                                                         int H, int K, const float2* __restrict__ twy) {
   __shared__ __align__(16) float2 ts[kMidChunk][kMidM];
   const int c = threadIdx.x & 31;
@@ -401,7 +399,7 @@ __global__ void __launch_bounds__(128) fno_dft_y_kernel(const float2* __restrict
         float2 v[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-          v[u] = ok && y0 + u * ns < ny ? __ldg(&a[(long)(yc + y0 + u * ns) * K * kFC]) : make_float2(0.f, 0.f);
+          v[u] = ok && y0 + u * ns < ny ? a[(long)(yc + y0 + u * ns) * K * kFC] : make_float2(0.f, 0.f);
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           if (y0 + u * ns >= ny) break;
@@ -429,7 +427,7 @@ __global__ void __launch_bounds__(128) fno_dft_y_kernel(const float2* __restrict
 // with F = R[mode] or (ADJ) its conjugate transpose; a thread takes one o of kMixB samples.
 constexpr int kMixB = 4;
 template <bool ADJ>
-__global__ void __launch_bounds__(256) fno_mix_kernel(const float2* __restrict__ X, float2* __restrict__ Y,
+__global__ void __launch_bounds__(256) fno_mix_kernel(const float2* X, float2* __restrict__ Y,
                                                        const float* __restrict__ R, int B, int K) {
   __shared__ float2 F[kFC][kFC + 1];
   __shared__ __align__(16) float2 xs[8 * kMixB][kFC];
@@ -477,7 +475,7 @@ __global__ void __launch_bounds__(256) fno_mix_kernel(const float2* __restrict__
 }
 
 // Inverse column DFT: thread (o) of column (b, kx) forms kMidY rows from all modes.
-__global__ void __launch_bounds__(128) fno_idft_y_kernel(const float2* __restrict__ Y, float2* __restrict__ A, int B,
+__global__ void __launch_bounds__(128) fno_idft_y_kernel(const float2* Y, float2* __restrict__ A, int B,
                                                          int H, int K, const float2* __restrict__ twy) {
   __shared__ __align__(16) float2 ts[2 * kFMaxK][kMidY];
   const int o = threadIdx.x & 31;
@@ -499,7 +497,7 @@ __global__ void __launch_bounds__(128) fno_idft_y_kernel(const float2* __restric
       float2 a[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u)
-        a[u] = mc + u * ns < M2 ? __ldg(&v[(long)(mc + u * ns) * K * B * kFC]) : make_float2(0.f, 0.f);
+        a[u] = mc + u * ns < M2 ? v[(long)(mc + u * ns) * K * B * kFC] : make_float2(0.f, 0.f);
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         if (mc + u * ns >= M2) break;
@@ -540,9 +538,9 @@ __global__ void __launch_bounds__(128) fno_idft_y_kernel(const float2* __restric
 // ---------------------------------------------------------------------------
 template <bool BWD, int T>
 __global__ void __launch_bounds__(T == 8 ? 256 : 512, T == 8 ? 2 : 1)
-    fno_row_kernel(float2* A, const float* __restrict__ vin, const float* __restrict__ Wl,
+    fno_row_kernel(float2* A, const float* vin, const float* __restrict__ Wl,
                    const float* __restrict__ wl, float* __restrict__ pre, float* __restrict__ out,
-                   const float* __restrict__ gpre, int W, int Wp, int K, float scale, int gelu_out, int next,
+                   const float* gpre, int W, int Wp, int K, float scale, int gelu_out, int next,
                    const float* __restrict__ tw) {
   constexpr bool TWS = T == 4;
   constexpr int OG = kFC / T, H4 = T / 4;  // channel groups; float4 per operand
@@ -680,7 +678,7 @@ __device__ __forceinline__ void fno_proj_weights(float* Q1t, float* q1s, float* 
 }
 
 // the tile's v planes (zero beyond the last group)
-__device__ __forceinline__ void fno_load_tile(float* vs, const float* __restrict__ v, long tile, long groups, int Wp) {
+__device__ __forceinline__ void fno_load_tile(float* vs, const float* v, long tile, long groups, int Wp) {
   const int n4 = Wp / 4, g = threadIdx.x % (kPT / 4);
   const long gg = tile * (kPT / 4) + g;
   const long r = (int)gg / n4;  // (a group has 6 kB of activations, so their number fits 31 bits)
@@ -714,7 +712,7 @@ __device__ __forceinline__ void fno_reduce_pred(float (&o)[3][8], float (*red)[3
 }
 
 // Inference: h = q std + mean (float4 per cell), one tile per block.
-__global__ void __launch_bounds__(kPN) fno_proj_kernel(const float* __restrict__ v, long groups, int W, int Wp,
+__global__ void __launch_bounds__(kPN) fno_proj_kernel(const float* v, long groups, int W, int Wp,
                                                        const float* __restrict__ Q1, const float* __restrict__ q1,
                                                        const float* __restrict__ Q2, const float* __restrict__ q2,
                                                        float4* __restrict__ out, float3 mean, float3 sd) {
@@ -774,7 +772,7 @@ struct FnoTrainSmem {
 };
 
 __global__ void __launch_bounds__(kPN, 2)
-    fno_proj_train_kernel(const float* __restrict__ v, const float4* __restrict__ h_target, long groups, int W, int Wp,
+    fno_proj_train_kernel(const float* v, const float4* h_target, long groups, int W, int Wp,
                           const float* __restrict__ Q1, const float* __restrict__ q1, const float* __restrict__ Q2,
                           const float* __restrict__ q2, float3 mean, float3 inv_std, float inv_count,
                           float* __restrict__ dv, float* __restrict__ dQ1, float* __restrict__ dq1,
@@ -957,7 +955,7 @@ __global__ void __launch_bounds__(kPN, 2)
 // take a quarter of a chunk's cells each, a thread 4 x 4 outputs (channels 8
 // apart, so a warp's float4 reads meet no bank twice): 64 FMA per 8 loads.
 constexpr int kWgX = 64, kWgP = kWgX + 4;
-__global__ void __launch_bounds__(256) fno_wgrad_kernel(const float* __restrict__ du, const float* __restrict__ v,
+__global__ void __launch_bounds__(256) fno_wgrad_kernel(const float* du, const float* v,
                                                         long rows, int Wp, float* __restrict__ dW,
                                                         float* __restrict__ db) {
   __shared__ __align__(16) float as[2 * kFC * kWgP];
@@ -977,8 +975,8 @@ __global__ void __launch_bounds__(256) fno_wgrad_kernel(const float* __restrict_
 #pragma unroll
     for (int q = 0; q < NL; ++q) {
       const long at = (r * kFC + lc + q * (kFC / NL)) * Wp + x;
-      na[q] = in ? ldg4(du + at) : make_float4(0.f, 0.f, 0.f, 0.f);
-      nb[q] = in ? ldg4(v + at) : make_float4(0.f, 0.f, 0.f, 0.f);
+      na[q] = in ? f4(du + at) : make_float4(0.f, 0.f, 0.f, 0.f);
+      nb[q] = in ? f4(v + at) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   };
   load(blockIdx.x);
@@ -1027,7 +1025,7 @@ __global__ void __launch_bounds__(256) fno_wgrad_kernel(const float* __restrict_
 
 // Lifting layer's gradient: dP[o][k] += sum du[o][x] xn[k][x], dp[o] += sum
 // du[o][x]; warp o of the block, lanes over x.
-__global__ void __launch_bounds__(1024) fno_lift_grad_kernel(const float* __restrict__ du, const float4* __restrict__ m,
+__global__ void __launch_bounds__(1024) fno_lift_grad_kernel(const float* du, const float4* m,
                                                              long rows, int W, int Wp, float3 mean, float3 inv_std,
                                                              float* __restrict__ dP, float* __restrict__ dp) {
   const int o = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1037,7 +1035,7 @@ __global__ void __launch_bounds__(1024) fno_lift_grad_kernel(const float* __rest
     const float* d = du + (r * kFC + o) * Wp;
     for (int x = lane; x < W; x += 32) {
       const float u = d[x];
-      const float4 c = __ldg(&m[r * W + x]);
+      const float4 c = m[r * W + x];
       a[0] = fmaf(u, (c.x - mean.x) * inv_std.x, a[0]);
       a[1] = fmaf(u, (c.y - mean.y) * inv_std.y, a[1]);
       a[2] = fmaf(u, (c.z - mean.z) * inv_std.z, a[2]);
@@ -1055,7 +1053,7 @@ __global__ void __launch_bounds__(1024) fno_lift_grad_kernel(const float* __rest
 
 // Filter gradient per kept mode: dR[mode][i][o] = s_kx sum_b conj(X[mode][b][i]) Xg[mode][b][o],
 // s_kx = (kx == 0 ? 1 : 2) / (H W).  One block of 32 x 32 threads per mode.
-__global__ void __launch_bounds__(1024) fno_rgrad_kernel(const float2* __restrict__ X, const float2* __restrict__ Xg,
+__global__ void __launch_bounds__(1024) fno_rgrad_kernel(const float2* X, const float2* Xg,
                                                          float* __restrict__ dR, int B, int K, float scale) {
   __shared__ float2 xs[kFC][kFC];
   __shared__ float2 gs[kFC][kFC];

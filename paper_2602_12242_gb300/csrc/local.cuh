@@ -30,12 +30,12 @@ __device__ __forceinline__ void neighbours(const float4* __restrict__ m, const G
                                            int j, int k, long idx, float3 mc, float3& xp, float3& xm, float3& yp,
                                            float3& ym, float3& zp, float3& zm) {
   const long sx = 1, sy = g.nx, sz = (long)g.nx * g.ny;
-  xp = (i + 1 < g.nx) ? f3(__ldg(&m[idx + sx])) : make_float3(mc.x - c.kdx * mc.z, mc.y, mc.z + c.kdx * mc.x);
-  xm = (i > 0) ? f3(__ldg(&m[idx - sx])) : make_float3(mc.x + c.kdx * mc.z, mc.y, mc.z - c.kdx * mc.x);
-  yp = (j + 1 < g.ny) ? f3(__ldg(&m[idx + sy])) : make_float3(mc.x, mc.y - c.kdy * mc.z, mc.z + c.kdy * mc.y);
-  ym = (j > 0) ? f3(__ldg(&m[idx - sy])) : make_float3(mc.x, mc.y + c.kdy * mc.z, mc.z - c.kdy * mc.y);
-  zp = (k + 1 < g.nz) ? f3(__ldg(&m[idx + sz])) : mc;
-  zm = (k > 0) ? f3(__ldg(&m[idx - sz])) : mc;
+  xp = (i + 1 < g.nx) ? f3(m[idx + sx]) : make_float3(mc.x - c.kdx * mc.z, mc.y, mc.z + c.kdx * mc.x);
+  xm = (i > 0) ? f3(m[idx - sx]) : make_float3(mc.x + c.kdx * mc.z, mc.y, mc.z - c.kdx * mc.x);
+  yp = (j + 1 < g.ny) ? f3(m[idx + sy]) : make_float3(mc.x, mc.y - c.kdy * mc.z, mc.z + c.kdy * mc.y);
+  ym = (j > 0) ? f3(m[idx - sy]) : make_float3(mc.x, mc.y + c.kdy * mc.z, mc.z - c.kdy * mc.y);
+  zp = (k + 1 < g.nz) ? f3(m[idx + sz]) : mc;
+  zm = (k > 0) ? f3(m[idx - sz]) : mc;
 }
 
 // The six neighbours of a cell.
@@ -105,7 +105,7 @@ template <bool DMI>
 __device__ __forceinline__ void local_terms(const float4* __restrict__ m, const float4* __restrict__ hd,
                                             const Grid& g, const LocalCoef& c, int i, int j, int k, long idx,
                                             float3 mc, float inv_ms, Terms& t) {
-  local_terms_v<DMI>(m, hd ? f3(__ldg(&hd[idx])) : make_float3(0.f, 0.f, 0.f), g, c, i, j, k, idx, mc, inv_ms, t);
+  local_terms_v<DMI>(m, hd ? f3(hd[idx]) : make_float3(0.f, 0.f, 0.f), g, c, i, j, k, idx, mc, inv_ms, t);
 }
 
 __device__ __forceinline__ float3 llg(const LocalCoef& c, float3 mc, float3 H) {
@@ -251,7 +251,7 @@ __device__ __forceinline__ void local_cell_v(const StageIO& io, const Grid& g, c
 template <int MODE, bool DMI>
 __device__ __forceinline__ void local_cell(const StageIO& io, const Grid& g, const LocalCoef& c, int i, int j, int k,
                                            long idx, int* flag) {
-  local_cell_v<MODE, DMI>(io, g, c, i, j, k, idx, io.hd ? f3(__ldg(&io.hd[idx])) : make_float3(0.f, 0.f, 0.f), flag);
+  local_cell_v<MODE, DMI>(io, g, c, i, j, k, idx, io.hd ? f3(io.hd[idx]) : make_float3(0.f, 0.f, 0.f), flag);
 }
 
 }  // namespace mx

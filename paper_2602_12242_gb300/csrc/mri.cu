@@ -33,8 +33,8 @@ constexpr double kAext[4][3] = {{0.0, 0.0, 0.0}, {kA21, 0.0, 0.0}, {kA31, kA32, 
 // interval's forcing r = wf f + w0 F0 + w1 F1 (F0, F1: those of the stages before, null
 // where there are none).  F and r: where f and r go (null: not kept).
 struct SlowIO {
-  const float4* __restrict__ m;
-  const float4* __restrict__ hd;
+  const float4* m;
+  const float4* hd;
   const float4* F0;
   const float4* F1;
   float4* F;
@@ -43,8 +43,8 @@ struct SlowIO {
 };
 template <bool DMI>
 __global__ void __launch_bounds__(256) mri_slow_kernel(SlowIO io, Grid g, LocalCoef c, int* flag) {
-  const float4* __restrict__ m = io.m;
-  const float4* __restrict__ hd = io.hd;
+  const float4* m = io.m;
+  const float4* hd = io.hd;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -68,11 +68,11 @@ __global__ void __launch_bounds__(256) mri_slow_kernel(SlowIO io, Grid g, LocalC
 
 // The fast step's stage data.
 struct FastIO {
-  const float4* __restrict__ u;  // stage input (stencil acts on it)
+  const float4* u;  // stage input (stencil acts on it)
   float4* __restrict__ v;        // fast step start; the step result replaces it (stage 2)
   float4* __restrict__ acc;      // stage 0: k1; stage 1 on: b1 k1 + b2 k2
   float4* __restrict__ out;      // stages 0, 1: next stage input
-  const float4* __restrict__ r;  // forcing
+  const float4* r;  // forcing
   float h;                       // fast step
 };
 
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(256) mri_fast_kernel(FastIO io, Grid g, LocalC
   if (i >= g.nx || j >= g.ny) return;
   const long idx = ((long)k * g.ny + j) * g.nx + i;
   const float3 uc = f3(io.u[idx]);
-  const float3 r = f3(__ldg(&io.r[idx]));
+  const float3 r = f3(io.r[idx]);
   const float3 v = STAGE == 0 ? uc : f3(io.v[idx]);
   const float3 a = STAGE == 0 ? make_float3(0.f, 0.f, 0.f) : f3(io.acc[idx]);
   const float ms = c.ms_map ? __ldg(&c.ms_map[idx]) : c.Ms;

@@ -136,7 +136,7 @@ template <int M> struct RowTw {
 // t = conj(W_2M^k) (X[k] - conj X[M-k]); element n of the inverse transform of Z
 // is cells 2n (real part) and 2n + 1 (imaginary part).
 template <int M, int R>
-__device__ __forceinline__ void xi_rows(float2* sm, const float2* __restrict__ w1, const Grid& g, int row0,
+__device__ __forceinline__ void xi_rows(float2* sm, const float2* w1, const Grid& g, int row0,
                                         const RowTw<M>& tw) {
   typedef RowShape<M, R> RS;
   typedef Line8<M> L;
@@ -191,14 +191,14 @@ __device__ __forceinline__ void xf_cell(float2* sm, int r, int i, float3 v) {
 
 // xf_cell for the cells of rows row0 .. row0 + R - 1 of Ms m in global memory.
 template <int M, int R, int NT>
-__device__ __forceinline__ void xf_stage(float2* sm, const float4* __restrict__ m, const Grid& g, float ms,
+__device__ __forceinline__ void xf_stage(float2* sm, const float4* m, const Grid& g, float ms,
                                          const float* __restrict__ ms_map, int row0) {
   const int total = min(R, g.ny * g.nz - row0) * g.nx;
 #pragma unroll 4
   for (int e = threadIdx.x; e < total; e += NT) {
     const int r = R == 1 ? 0 : e / g.nx, i = e - r * g.nx;
     const long idx = (long)row0 * g.nx + e;
-    const float4 a = __ldg(&m[idx]);
+    const float4 a = m[idx];
     const float s = ms_map ? __ldg(&ms_map[idx]) : ms;
     xf_cell<M, R>(sm, r, i, make_float3(s * a.x, s * a.y, s * a.z));
   }

@@ -224,3 +224,29 @@ def test_output_does_not_depend_on_the_batch_size(nx, ny, K):
     full = net.forward(dev4(m)).cpu()
     for b in (1, 2, 4, 5, 8):
         assert torch.equal(net.forward(dev4(m[3:3 + b])).cpu(), full[3:3 + b]), b
+
+
+@pytest.mark.parametrize("nx,ny,K,B", [(40, 24, 8, 5), (24, 20, 8, 7), (37, 26, 5, 5), (24, 16, 4, 2), (24, 16, 4, 9)])
+def test_short_chains_of_calls_match_oracle(nx, ny, K, B):
+    """Every kernel of the batch column pass, of the row passes and of the weight gradients has at most a
+    block per SM, so each starts while the one before runs: calls on three inputs in turn, outputs and
+    gradients at the tolerances of the tests above."""
+    flat = params_for(K, 41)
+    net = make_net(nx, ny, K, B, flat)
+    ms = [fields(B, ny, nx, q) for q in (42, 43, 44)]
+    tg = [(fields(B, ny, nx, q) * 1.5 * STATS[9:12] + STATS[6:9]).astype(np.float32).astype(np.float64)
+          for q in (45, 46, 47)]
+    dm, dt = [dev4(m) for m in ms], [dev4(t) for t in tg]
+    hs = [net.forward(m).clone() for _ in range(2) for m in dm]
+    gs = [net.loss_grad(m, t)[1].clone() for _ in range(2) for m, t in zip(dm, dt)]
+    offs = np.cumsum([0] + [int(np.prod(s)) for s in fno.param_shapes(K)])
+    for q in range(3):
+        ref = oracle_h(flat, ms[q], K)
+        x = fno.to_nchw((ms[q] - STATS[0:3]) / STATS[3:6])
+        t = fno.to_nchw((tg[q] - STATS[6:9]) / STATS[9:12])
+        g_ref = fno.loss_and_grad(torch.from_numpy(flat), x, t, K)[1].numpy()
+        for h, g in ((hs[q], gs[q]), (hs[q + 3], gs[q + 3])):
+            assert rel_l2(h.cpu().numpy()[:, 0, :, :, :3], ref) <= 2e-5
+            g = g.cpu().numpy().astype(np.float64)
+            for i in range(len(offs) - 1):
+                assert rel_l2(g[offs[i]:offs[i + 1]], g_ref[offs[i]:offs[i + 1]]) <= 1e-4, fno.param_shapes(K)[i]

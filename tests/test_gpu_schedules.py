@@ -216,3 +216,52 @@ def test_film_kernels_of_many_columns_match_generic_passes(nx, ny):
     assert ctx.kernel_name("yz_fused") == ("yz2d_wide_kernel" if ny > 128 else "yz2d_kernel")
     ref, _ = field(c, demag_path=_lib.MX_DEMAG_GENERIC)
     assert rel_l2(h, ref) <= TOL
+
+
+# Deep grids whose row kernels are at most a block per SM, so that the y pass starts while they run: one
+# field after another and steps, against the generic passes.  (The spectrum of the field or stage before
+# is an error of order one in H, 1e-3 of m per step here.)
+@pytest.mark.parametrize("shape", [(26, 25, 20), (28, 24, 25), (64, 17, 17), (12, 20, 25), (16, 33, 18), (40, 17, 17)])
+def test_deep_grids_of_few_rows_match_generic_passes(shape):
+    from paper_2602_12242_gb300 import MX_TERM_DEMAG, _lib
+    from paper_2602_12242_gb300.solver import from_dev4, to_dev4
+    c = cfg_of(nx=shape[0], ny=shape[1], nz=shape[2], dx=2e-9, dy=2.5e-9, dz=3e-9)
+    ms = [to_dev4(np.asarray(random_m(c, q), np.float32)) for q in (41, 42, 43)]
+    out = []
+    for path in (_lib.MX_DEMAG_AUTO, _lib.MX_DEMAG_GENERIC):
+        ctx = context(c, demag_path=path)
+        if path == _lib.MX_DEMAG_AUTO:
+            assert ctx.kernel_name("y_fwd") == "deep_yf_kernel" and ctx.kernel_name("x_inv_local") == "xr_kernel"
+        got = []
+        for _ in range(3):
+            got += [ctx.heff(m, terms=MX_TERM_DEMAG) for m in ms] + [ctx.llg_rhs(m) for m in ms]
+        for method in ("rk4", "euler"):
+            for n in (2, 5):
+                m = ms[0].clone()
+                ctx.rk_step(m, n, 1e-14, method)
+                got.append(m)
+        ctx.sync()
+        out.append([from_dev4(x) for x in got])
+    for a, b in zip(*out):
+        assert rel_l2(a, b) <= TOL
+
+
+# Few-layer and one-layer grids of at most a block per SM in every kernel: the inverse x pass, on both
+# layouts of the spectrum, starts while the y/z kernel runs, and the right-hand side's local kernel while
+# the inverse x pass does
+@pytest.mark.parametrize("shape", [(100, 128, 5), (50, 64, 14), (60, 100, 4), (40, 20, 2), (20, 30, 1), (100, 16, 9)])
+def test_short_chains_of_fields_match_generic_passes(shape):
+    from paper_2602_12242_gb300 import MX_TERM_DEMAG, _lib
+    from paper_2602_12242_gb300.solver import from_dev4, to_dev4
+    c = cfg_of(nx=shape[0], ny=shape[1], nz=shape[2], dx=2e-9, dy=2.5e-9, dz=3e-9)
+    ms = [to_dev4(np.asarray(random_m(c, q), np.float32)) for q in (41, 42, 43)]
+    out = []
+    for path in (_lib.MX_DEMAG_AUTO, _lib.MX_DEMAG_GENERIC):
+        ctx = context(c, demag_path=path)
+        got = []
+        for _ in range(3):
+            got += [ctx.heff(m, terms=MX_TERM_DEMAG) for m in ms] + [ctx.llg_rhs(m) for m in ms]
+        ctx.sync()
+        out.append([from_dev4(x) for x in got])
+    for a, b in zip(*out):
+        assert rel_l2(a, b) <= TOL
