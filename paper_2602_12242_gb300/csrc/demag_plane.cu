@@ -266,7 +266,7 @@ __device__ __forceinline__ void xil_cells(const float2* sm, int P, int NT, const
     const float2 hx = L[0], hy = L[P], hz = L[2 * P];
     const float3 hdv = (i & 1) ? make_float3(hx.y, hy.y, hz.y) : make_float3(hx.x, hy.x, hz.x);
     const int y = y0 + r;
-    local_cell_v<MODE, DMI>(io, g, c, i, y, z, ((long)z * g.ny + y) * g.nx + i, hdv, flag);
+    local_cell_v<MODE, DMI, true>(io, g, c, i, y, z, ((long)z * g.ny + y) * g.nx + i, hdv, flag);
   }
 }
 

@@ -22,7 +22,7 @@
 
 namespace mx {
 
-template <int MODE, bool DMI>
+template <int MODE, bool DMI, bool FAR>
 __global__ void __launch_bounds__(256) local_kernel(StageIO io, Grid g, LocalCoef c, int* flag) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(256) local_kernel(StageIO io, Grid g, LocalCoe
   pdl_wait();
   if (i >= g.nx || j >= g.ny) return;
   const long idx = ((long)k * g.ny + j) * g.nx + i;
-  local_cell<MODE, DMI>(io, g, c, i, j, k, idx, flag);
+  local_cell<MODE, DMI, FAR>(io, g, c, i, j, k, idx, flag);
 }
 
 __global__ void normalize_kernel(float4* m, long n, int* flag) {
@@ -126,10 +126,10 @@ LocalCoef local_coef_from(const mx_params& p, const float* ms_map, const float* 
 template <int MODE>
 static void launch_local(bool dmi, dim3 grid, dim3 block, cudaStream_t st, const StageIO& io, const Grid& g,
                          const LocalCoef& c, int* flag) {
-  if (dmi)
-    launch_pdl(local_kernel<MODE, true>, grid, block, 0, st, io, g, c, flag);
-  else
-    launch_pdl(local_kernel<MODE, false>, grid, block, 0, st, io, g, c, flag);
+  // with a demag field, its kernels come between what wrote io.m and this
+  auto k = io.hd ? (dmi ? local_kernel<MODE, true, true> : local_kernel<MODE, false, true>)
+                 : (dmi ? local_kernel<MODE, true, false> : local_kernel<MODE, false, false>);
+  launch_pdl(k, grid, block, 0, st, io, g, c, flag);
 }
 
 static void local_dims(const Grid& g, dim3& grid, dim3& block) {

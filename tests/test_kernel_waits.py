@@ -16,8 +16,9 @@ import paper_2602_12242_gb300
 CSRC = os.path.join(os.path.dirname(paper_2602_12242_gb300.__file__), "csrc")
 SRC = os.path.join(CSRC, "cnn.cu")
 
-# tables, the tensor, networks' parameters (last written before the kernel before) and material maps
-CONSTANTS = {"twM", "twP", "twH", "twPy", "twL", "tw", "twx", "twy", "twz", "agl", "nhat", "nhk", "n", "t", "Rm", "R",
+# tables, the tensor, networks' parameters and the forward pass's pre-activations (last written before
+# the kernel before) and material maps
+CONSTANTS = {"gpre", "twM", "twP", "twH", "twPy", "twL", "tw", "twx", "twy", "twz", "agl", "nhat", "nhk", "n", "t", "Rm", "R",
              "Wl", "wl", "Q1", "q1", "Q2", "q2", "p.bias", "ms_map", "c.ms_map", "c.ku_map", "c.axis_map"}
 # (kernels launched after the one before has ended)
 ORDINARY = {"yzh_kernel"}
@@ -74,5 +75,5 @@ def test_non_coherent_loads_read_only_constants():
                 text = text.replace(body, "")
         for m in re.finditer(r"(?:__ldg|ldg4)\((?:reinterpret_cast<const float[24]\*>\()?&?([\w.]+)", text):
             if m[1] in ("const", "p") or "ldg4(a +" in text[m.start():m.end() + 3]:
-                continue  # (ldg4's own definition; twiddle rows)
+                continue  # (ldg4's own definition, load3<FAR>'s; twiddle rows)
             assert m[1] in CONSTANTS, (os.path.basename(f), m[1], text[m.start():m.end() + 20])
