@@ -18,7 +18,8 @@
 //   backward-W  dW[tap] = sum over cells of dY (x) x_shifted(tap)
 // Every convolution and weight gradient is a tcgen05 (BF16 in, FP32 accumulator
 // in tensor memory) kernel of three roles: a producer warp issues the bulk
-// copies, one thread the MMAs, eight warps run the epilogue of the tile before;
+// copies, one thread the MMAs, eight or sixteen warps (four in the weight
+// gradient) run the epilogue of the tile before;
 // they meet at mbarriers only (every wait bounded; one that runs out sets
 // kFlagTimeout and its role stops).  The last layer's epilogue denormalises, or
 // in training forms the loss and its gradient.
@@ -114,8 +115,8 @@ struct ConvArgs {
 // CTA walks z fastest, so each tile brings one new plane; the planes of tile t +
 // 1 arrive and its MMAs start while the epilogue of tile t runs (two accumulators
 // in tensor memory).
-// Bound: the MMAs, at 60 to 80 cycles each whatever N <= 64 is (their A operand is 4
-// KB of shared memory), and for 64 output channels the issue slots of the epilogue's
+// Bound: the MMAs, at about 80 cycles each whatever N <= 64 is (their A operand is 4
+// KB of shared memory; 78 over a whole launch of 64 -> 32 channels, 85 of 32 -> 3), and for 64 output channels the issue slots of the epilogue's
 // erf.  Measured forward at 64 samples of 64x64x4, with the kernel before in brackets
 // (256 threads copied three planes per tile with cp.async, waited for the MMAs and
 // ran the epilogue in turn): 3 -> 32 channels 98 us (230), 32 -> 64 167 (362), 64 ->
@@ -402,8 +403,8 @@ __global__ void __launch_bounds__(ConvTc<CIN, COUT>::threads, 1)
 // The chains are added in FP32 in ws[(dz 3 + dy) CR + cr][(s, cs)], lanes next to
 // each other.  Bound: the MMAs' operand reads (6 KB per MMA at N = 64) and L2.
 // Measured at 64 samples of 64x64x4, with the kernel before in brackets (a (dz, dy)
-// per block, a tap per MMA, copies and MMAs in turn): 64 -> 32 and 32 -> 64 115 us
-// each (863, 600), 3 -> 32 and 32 -> 3 89 each (315, 452).  A CTA per SM with five or
+// per block, a tap per MMA, copies and MMAs in turn): 64 -> 32 and 32 -> 64 110 us
+// each (863, 600), 3 -> 32 and 32 -> 3 88 each (315, 452).  A CTA per SM with five or
 // four of the nine (dz, dy), planes of R kept in a ring: 131 and 101.
 // ---------------------------------------------------------------------------
 constexpr int kTX = 16, kTY = 8;  // tile (cells)

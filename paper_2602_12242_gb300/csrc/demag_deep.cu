@@ -24,12 +24,13 @@
 // thread holds the three components of its wavenumbers and multiplies in
 // registers.  Neighbouring lanes take neighbouring kx (T of them contiguous).
 //
-// Bound: instruction issue (128^3: 72 M warp instructions in zc, half of the
-// issue slots) and the latency of the phases between barriers; a first version
+// Bound: instruction issue (128^3: 76 M warp instructions in zc, 57 % of the
+// issue slots), shared memory (51 % of its wavefronts) and the latency of the
+// phases between barriers; a first version
 // that kept lines in natural order moved every value through shared memory 14
 // times where this one does 5 (9 in zc of long lines).  Measured at 128^3 (256^3
-// padded), against the size-generic passes: yf 37 us (266), zc 119 us (884; 136
-// in natural order), yi 43 us (330).
+// padded), against the size-generic passes: yf 36 us (266), zc 113 us (884; 136
+// in natural order), yi 41 us (330).
 #include <math.h>
 
 #include "common.cuh"

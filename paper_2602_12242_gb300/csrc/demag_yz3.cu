@@ -11,18 +11,19 @@
 // components in registers (zcol.cuh), one kz parity where the block has the
 // threads for both, else both in turn.  Inverse y is the mirror image: even +
 // W_Py^-y odd.  The zero halves along y and z are never formed, and the block
-// meets eight barriers, where the block-wide radix passes of yz_fused_kernel
+// meets five barriers (seven with the split z stage), where the block-wide radix passes of yz_fused_kernel
 // meet two per pass and transform the padding too.  The tensor octant is in
 // plane_octant_index order (six components innermost), so a column's entry is
 // three 8-byte loads and neighbouring columns are contiguous.
 //
 // Bound: the latency of that chain (load, two line FFTs, column, store) at two
-// to four blocks per SM, and on large grids instruction issue (60 % at 640x160x4).
+// to four blocks per SM, and on large grids instruction issue (58 % of its slots at 640x160x4).
 // Measured (one evaluation, kernel alone): 32x32x4 14.1 -> 3.9 us and 201x77x3 73.4
 // -> 9 us against yz_fused_kernel; 640x160x4 107 -> 42 us (49 with divisions by
 // run-time sizes in the load and store loops), 256x256x4 32 -> 16 us and 256x256x8
 // 42 -> 35 us against the four-CTA plane kernel, whose cluster barriers and small
-// shares of a plane cost more than they save where a plane fits one block.
+// shares of a plane cost more than they save where a plane fits one block (but for
+// grids with at most one kx column to two SMs, quad_first in demag_plane.cu).
 #include <math.h>
 
 #include "common.cuh"

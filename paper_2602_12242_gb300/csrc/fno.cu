@@ -533,9 +533,10 @@ __global__ void __launch_bounds__(128) fno_idft_y_kernel(const float2* Y, float2
 // FMA.  T = 8 for batches: a float4 load occupies the load path for four cycles
 // whatever its addresses, so 4 x 4 tiles are bound by it at half the FMA rate.
 // T = 4 with the twiddle rows in shared memory where there are few rows, for the
-// shorter chain.  Bound: for batches FP32 issue (of 50 M warp instructions a
-// pass of 32 fields of 160 x 40, 19 M are the products, the rest mostly erf and
-// exp); 53 us where the lane-per-channel kernel took 85.  Not kept: persistent
+// shorter chain.  Bound: for batches FP32 issue (a pass of 32 fields of 160 x 40
+// is 34.9 M warp instructions at 63 % of the issue slots, 16.4 M of them the FMAs of
+// the products and of the row DFT); 51 us in the chain of a training step where the
+// lane-per-channel kernel took 85.  Not kept: persistent
 // blocks with two row buffers (97 us at 8 warps per SM, 71 with one buffer).
 // ---------------------------------------------------------------------------
 template <bool BWD, int T>
