@@ -190,8 +190,8 @@ mx_status mx_llg_rhs(mx_ctx *ctx, const float *m, float *dmdt, mx_stream_t strea
 /* Advance m in place by nsteps steps of size dt [s] with MX_RK4 (four
  * right-hand-side evaluations, every stage input and the result
  * renormalised) or MX_EULER.  m is normalised on entry.  The first call for
- * a given (m, dt, method, nsteps > 1) captures one step into a CUDA graph
- * that later calls replay.  Non-finite values set a device flag that
+ * a given (m, dt, method) captures one step (MX_EULER: two, and one for an
+ * odd count) into a CUDA graph that later calls replay.  Non-finite values set a device flag that
  * mx_sync reports. */
 mx_status mx_rk_step(mx_ctx *ctx, float *m, int nsteps, double dt, int method,
                      mx_stream_t stream);
